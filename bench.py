@@ -39,19 +39,18 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "X-drop GCUPS (computed cells), batched vs plain launch; serving p50/p99 ms"
-# From one ncu capture of the level-2 kernel (k_group16<4>, the packed
-# 16-bit form) on the 24,000-pair lognormal batch (48,000 extensions
-# started):
+# From one ncu capture of the level-2 kernel (k_diag16<4, 1, 16>, the packed 16-bit
+# form) on the 24,000-pair lognormal batch (48,000 extensions started):
 #   bytes     dram__bytes_read.sum + dram__bytes_write.sum of the launch,
 #             scaled to a launch by the extensions it starts;
 #   fma_share the share of its executed warp instructions that issue to the
 #             FMA pipe (IMAD, from sass__inst_executed_per_opcode), the rest
 #             going to the ALU pipe or to pipes that are not near a limit.
 # Reported only while the kernel's sources are the ones captured.
-PROFILED = {"level": 2, "bytes": 114.171904e6 + 9.26592e6, "items": 48_000,
-            "fma_share": 6171644505 / 20159301634,
-            "sources": ("xdrop_group16.cu", "packed16.cuh", "logan_dev.cuh", "internal.h"),
-            "sha1": "018a8d6b1c9b48304bbd4acb8c1f2e36f6878139"}
+PROFILED = {"level": 2, "bytes": 113.526016e6 + 9.176064e6, "items": 48_000,
+            "fma_share": 3756977838 / 12909251907,
+            "sources": ("xdrop_diag16.cu", "diag16.cuh", "logan_dev.cuh", "internal.h"),
+            "sha1": "fe1df1c0ebb74f32418bb8e80f06b5f22b41b82c"}
 OPS_PER_CELL_AFFINE = 12  # Gotoh per cell: compare, diag add, E: 2 adds + max, F: 2 adds + max, 2 max, X-drop compare, select
 # The scope table's count for the linear recurrence, per cell: substitution
 # select, diag + substitution, max(up, left), + gap and max with the diagonal

@@ -455,20 +455,23 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
 #define LOGAN_OPT_PACKED16 11    /* 1 (default): a window level that has a
                                     packed form (two 16-bit cells per 32-bit
                                     register) runs it when the call's scoring
-                                    and X provably fit 16 bits --
-                                    128 * (Xmax + 2*max(match,0) + |gap| + 2)
-                                    + 31 <= 32767 and 128 * (|mismatch| +
-                                    |gap| + 2*max(match,0) + 2) <= 16383, Xmax
-                                    the largest X that can reach the level
+                                    and X provably fit 16 bits: for the
+                                    linear levels when some K in {64, 32, 16,
+                                    8, 4} has, with mp = max(match, 0) and
+                                    D = K*|gap| + mp*(K/2 + 1),
+                                    32 * (D + Xmax + mp + 1) + 32 <= 32767 and
+                                    32 * (D + 2*|gap| + 2*mp + 2) + 64 <= 32767,
+                                    Xmax the largest X that can reach the level
                                     (the scalar X, or the X-class bounds of
                                     the start-level table when X is per pair
-                                    or a start level is forced); otherwise,
-                                    or with 0, the 32-bit form.  Results are
-                                    identical either way.  The affine call's
-                                    windows of 128, 256 and 512 rows follow
-                                    the same option with |gap_open| +
-                                    |gap_extend| for |gap| and 2*|gap_extend|
-                                    in the second bound. */
+                                    or a start level is forced); for the affine
+                                    call's windows of 128, 256 and 512 rows
+                                    when 128 * (Xmax + 2*mp + |gap_open| +
+                                    |gap_extend| + 2) + 31 <= 32767 and
+                                    128 * (|mismatch| + |gap_open| +
+                                    2*|gap_extend| + 2*mp + 2) <= 16383;
+                                    otherwise, or with 0, the 32-bit form.
+                                    Results are identical either way. */
 #define LOGAN_OPT_AFFINE_PACKED 12 /* read-only: bit l set when affine window
                                     level l (64, 128, 256, 512 rows) ran in
                                     its packed 16-bit form in the context's

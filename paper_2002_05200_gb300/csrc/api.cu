@@ -41,6 +41,11 @@ struct AuxSet {
     cudaEvent_t fork = nullptr;
     cudaEvent_t join[kUnits] = {};
 };
+// the levels that run packed in a call (bit l: level l) and their constants
+struct PackedPlan {
+    uint32_t levels = 0u;
+    DiagArgs args[kNumLevels];
+};
 inline size_t up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct GraphEntry {
@@ -239,11 +244,11 @@ void default_table(LevelTable& t) {
 }
 
 int launch_unit(logan_ctx* c, int u, const KernelArgs& ka, int phase, cudaStream_t s,
-                uint32_t packed) {
+                const PackedPlan& pk) {
     cudaError_t e;
-    if (u < kNumLevels && ((packed >> u) & 1u)) {
+    if (u < kNumLevels && ((pk.levels >> u) & 1u)) {
         const int grid = c->num_sms * std::max(1, c->packed_blocks_per_sm[u]);
-        e = launch_packed_level_persistent(u, ka, grid, phase, s);
+        e = launch_packed_level_persistent(u, ka, pk.args[u], grid, phase, s);
     } else if (u >= kNumLevels) {
         const int l = u - kNumLevels;
         const int grid = c->num_sms * std::max(1, c->twin_blocks_per_sm[l]);
@@ -289,21 +294,16 @@ AuxSet* aux_for(logan_ctx* c, cudaStream_t s) {
 }
 
 // Levels that run in their packed 16-bit form in this call: those with a
-// packed kernel, when
-//   128 * (Xmax + 2*max(match,0) + |gap| + 2) + 31 <= 32767  and
-//   128 * (|mismatch| + |gap| + 2*max(match,0) + 2) <= 16383,
-// Xmax the largest X that can reach the level: the scalar X when there is
-// no per-pair X and no forced start level, else the upper bound of every X
+// packed kernel whose bounds (xdrop_diag16.cu) hold for the scoring and the
+// largest X that can reach the level -- the scalar X when there is no
+// per-pair X and no forced start level, else the upper bound of every X
 // class whose start level is at or below it (items only move to wider
-// levels).  These bounds keep every 16-bit half inside [0, 65536) through
-// the kernel's additions (xdrop_group16.cu).
-uint32_t packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int32_t* Xs,
-                         const LevelTable& tab, int64_t force) {
-    if (!c->packed16) return 0u;
+// levels).
+PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int32_t* Xs,
+                           const LevelTable& tab, int64_t force) {
+    PackedPlan pk;
+    if (!c->packed16) return pk;
     static const int64_t upper[kXClasses] = {15, 35, 75, 150, 300, 700, 2000, int64_t(1) << 29};
-    const int64_t mp = std::max<int64_t>(sc.match, 0);
-    const int64_t ag = -int64_t(sc.gap), am = sc.mismatch < 0 ? -int64_t(sc.mismatch) : sc.mismatch;
-    uint32_t mask = 0u;
     for (int l = 0; l < kNumLevels; ++l) {
         if (!packed_level(l) || l > tab.max_level) continue;
         int64_t xmax = 0;
@@ -315,11 +315,9 @@ uint32_t packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int32_
             for (int k = 0; k < kXClasses; ++k)
                 if (tab.lv[k] <= l) xmax = std::max(xmax, upper[k]);
         }
-        constexpr int64_t S = 128;  // score scale of the packed keys
-        if (S * (xmax + 2 * mp + ag + 2) + 31 <= 32767 && S * (am + ag + 2 * mp + 2) <= 16383)
-            mask |= 1u << l;
+        if (packed_plan(sc, xmax, &pk.args[l])) pk.levels |= 1u << l;
     }
-    return mask;
+    return pk;
 }
 
 // Affine levels that run in their packed 16-bit form in this call: those
@@ -457,7 +455,8 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     }
     ka.mig_slot = reinterpret_cast<int32_t*>(ws + L.mig_slot);
     const int64_t forced = c->force_level >= 0 ? std::min<int64_t>(c->force_level, maxl) : -1;
-    const uint32_t packed = (aff || plain) ? 0u : packed16_levels(c, sc, X, Xs, tab, forced);
+    const PackedPlan packed =
+        (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced);
     if (aff) {
         // affine levels, narrowest first (each receives the bands that
         // outgrew the previous one), then the rejected items, then combine
@@ -565,7 +564,7 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         ci.p1_levels = p1_levels;
         ci.p2_levels = p2_levels;
         ci.plain = plain != 0;
-        ci.packed = packed;
+        ci.packed = packed.levels;
         c->timed_calls += 1;
         c->timing_pending = true;
     }

@@ -64,16 +64,32 @@ __device__ __forceinline__ int escalate_queue(const KernelArgs& ka, int level, b
     return (twin && nl < kTwinLevels) ? twin_queue(nl) : nl;
 }
 
+// Constants of a packed launch (xdrop_diag16.cu), from the scoring and the
+// largest X that can reach the level.
+struct DiagArgs {
+    int gap;     // gap score per base (<= 0)
+    int mp;      // max(match, 0)
+    int step;    // theta's growth per anti-diagonal: 32 * -gap
+    int floor;   // smallest key (a dead one)
+    int iters;   // loop iterations (two anti-diagonals each) between renormalisations
+    int unit;    // match - mismatch == 2 * (mismatch - 2 gap): one multiply-add per substitution
+    // multipliers of a mask bit at position p: mismatch - 2 gap and match -
+    // mismatch in key units, divided by 2^p
+    uint32_t cb[6], cf[6];
+};
+
 // extension kernels (xdrop_group.cu / xdrop_cta.cu / xdrop_ring.cu)
 cudaError_t launch_warp_level_persistent(int level, const KernelArgs& ka, int grid, int phase,
                                          cudaStream_t s);
 cudaError_t launch_warp_level_plain(int level, const KernelArgs& ka, cudaStream_t s);
 int warp_level_blocks_per_sm(int level);
-// packed 16-bit form of a register level (xdrop_group16.cu): same queues,
+// packed 16-bit form of a register level (xdrop_diag16.cu): same queues,
 // results and band-state records as the level's 32-bit kernel
 bool packed_level(int level);
-cudaError_t launch_packed_level_persistent(int level, const KernelArgs& ka, int grid, int phase,
-                                           cudaStream_t s);
+// the constants for this scoring and X, false when the scores do not fit
+bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da);
+cudaError_t launch_packed_level_persistent(int level, const KernelArgs& ka, const DiagArgs& da,
+                                           int grid, int phase, cudaStream_t s);
 int packed_level_blocks_per_sm(int level);
 // level k's one-warp form (k < kTwinLevels), persistent over twin_queue(k)
 cudaError_t launch_twin_persistent(int level, const KernelArgs& ka, int grid, int phase,

@@ -1,5 +1,5 @@
-// Shared pieces of the packed 16-bit kernels (xdrop_group16.cu: linear
-// gaps; xdrop_affine16.cu: affine gaps): the key encoding, the per-unit
+// Shared pieces of the packed 16-bit kernels (xdrop_affine16.cu: affine
+// gaps; the packed windows of xdrop_matrix.cu): the key encoding, the per-unit
 // state, the code bit planes and the reductions.  Two band rows share one
 // 32-bit register as 16-bit keys 32768 + 128*u + (31 - k) (u the score
 // minus the anti-diagonal's pruning threshold, k the row within its

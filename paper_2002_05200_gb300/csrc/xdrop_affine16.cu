@@ -6,8 +6,7 @@
 // sweep, X-drop rule and band trimming (Sec. III-A, Algorithms 1 and 2;
 // other scoring schemes are the paper's future work, Sec. VIII) -- the
 // computation of the 32-bit affine kernel (xdrop_affine.cu), with the same
-// results.  Layout and keys as the packed linear kernel (xdrop_group16.cu,
-// packed16.cuh): lane g of a unit of G lanes owns window rows g*32 + k,
+// results.  Layout and keys (packed16.cuh): lane g of a unit of G lanes owns window rows g*32 + k,
 // register h holds rows h and h + 16, a live value is the key
 // 32768 + 128*u + (31 - k) with u = S - T_d (T_d = best_{<d} - X), DEAD =
 // 16384.  H on d-2 / d-1 / d lives in three register arrays that rotate;
