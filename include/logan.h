@@ -441,22 +441,23 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     0: level after level on the caller stream */
 #define LOGAN_OPT_LONG_ITEM 10   /* extensions starting at window levels 0-3
                                     run either several to a warp (most) or
-                                    in the level's latency form: one to a
-                                    warp with the same window (fewer
+                                    in the level's latency form: one (in a
+                                    small batch up to four) to a warp with
+                                    a window at least as wide (fewer
                                     instructions per anti-diagonal: what a
                                     long extension, which a batch waits for,
                                     or a batch too small to fill the GPU
-                                    needs).  v >= 0: latency form when
+                                    needs; level 4 has one too when packed).  v >= 0: latency form when
                                     m + n >= v; -1: never; -2 (default):
                                     automatic -- every item when the batch
                                     has at most 32 items per SM, else
-                                    m + n >= 65536.  Results never depend on
+                                    m + n >= 131072.  Results never depend on
                                     it. */
 #define LOGAN_OPT_PACKED16 11    /* 1 (default): a window level that has a
                                     packed form (two 16-bit cells per 32-bit
                                     register) runs it when the call's scoring
                                     and X provably fit 16 bits: for the
-                                    linear levels when some K in {64, 32, 16,
+                                    linear levels 0-6 when some K in {64, 32, 16,
                                     8, 4} has, with mp = max(match, 0) and
                                     D = K*|gap| + mp*(K/2 + 1),
                                     32 * (D + Xmax + mp + 1) + 32 <= 32767 and
@@ -601,7 +602,7 @@ int logan_autotune_save(const logan_ctx_t *ctx, const char *path);
  * all pinned.  The server uses the context exclusively (graphs, timing and
  * concurrent levels off: each request runs on its slot's stream;
  * LOGAN_OPT_LONG_ITEM set per request: 65536 while at most 8 requests are
- * in flight, else -1) until logan_server_destroy, which restores those
+ * in flight, else 131072) until logan_server_destroy, which restores those
  * four options; do not call other functions on that context
  * meanwhile.  The slots overlap only as far as the device's hardware work
  * queues allow: set CUDA_DEVICE_MAX_CONNECTIONS (up to 32) to at least

@@ -24,6 +24,9 @@ constexpr int kEvSets = 32;        // timed calls whose events are kept
 // Launch units: the window levels (0 .. kNumLevels-1), then the latency
 // forms of levels 0 .. kTwinLevels-1 (unit kNumLevels + k).
 constexpr int kUnits = kNumLevels + kTwinLevels;
+// one stream per unit, one for the latency form of the widest level that has
+// one without a queue of its own (kTwinLevels)
+constexpr int kStreams = kUnits + 1;
 inline int unit_queue(int u) { return u < kNumLevels ? u : twin_queue(u - kNumLevels); }
 inline int unit_level(int u) { return u < kNumLevels ? u : u - kNumLevels; }
 
@@ -37,9 +40,9 @@ constexpr int kEvPerSet = 4 * kUnits + 4;
 // Streams on which the start queues of one caller stream run concurrently.
 struct AuxSet {
     cudaStream_t main = nullptr;
-    cudaStream_t st[kUnits] = {};
+    cudaStream_t st[kStreams] = {};
     cudaEvent_t fork = nullptr;
-    cudaEvent_t join[kUnits] = {};
+    cudaEvent_t join[kStreams] = {};
 };
 // the levels that run packed in a call (bit l: level l) and their constants
 struct PackedPlan {
@@ -80,6 +83,7 @@ struct logan_ctx {
     // call's scoring and X provably fit (see packed16_levels), 0 = never
     int64_t packed16 = 1;
     int packed_blocks_per_sm[kNumLevels] = {};
+    int latency_blocks_per_sm[kLatencyLevels][3] = {};  // 1, 2, 4 extensions per warp
     int8_t next_level[kNumLevels] = {};
     // timing: the events of the last kEvSets timed calls (ring)
     cudaEvent_t evs[kEvSets][kEvPerSet] = {};
@@ -243,12 +247,41 @@ void default_table(LevelTable& t) {
     t.max_level = kNumLevels - 1;
 }
 
+// Extensions per warp of a packed latency form.  Few items (or the long ones
+// of a batch): one, the shortest step.  A small batch with more items than
+// four warps per SM would queue for the schedulers with one per warp: two or
+// four share a warp's step (16 pairs of 2 kbp: 0.28 / 0.32 / 0.40 ms with 1 / 2 / 4
+// per warp; 1,000 pairs: 0.57 / 0.53 / 0.50 ms).
+int latency_units(const logan_ctx* c, uint32_t n_items, uint32_t long_min) {
+    if (long_min != 0u) return 1;
+    const uint32_t sms = uint32_t(c->num_sms);
+    return n_items <= 4u * sms ? 1 : n_items <= 8u * sms ? 2 : 4;
+}
+
+// The latency form of `level`.  all: it runs every item of the level; else the
+// few long ones, with one block per SM (608 extensions): more blocks, mostly
+// without an item, keep the other forms' blocks from their SMs (20,000 pairs
+// of 5 kbp, none long: 7.1 ms with three, 6.8 with one; uneven pairs
+// up to 1 Mbp 236 and 227 ms).
+int launch_latency(logan_ctx* c, int level, int queue, int units, bool all, const KernelArgs& ka,
+                   int phase, cudaStream_t s, const PackedPlan& pk) {
+    const int k = units == 4 ? 2 : units - 1;
+    const int most = std::max(1, c->latency_blocks_per_sm[level][k]);
+    const int grid = c->num_sms * (all ? most : 1);
+    return launch_packed_latency(level, queue, units, ka, pk.args[level], grid, phase, s) ==
+                   cudaSuccess
+               ? LOGAN_OK
+               : LOGAN_ECUDA;
+}
+
 int launch_unit(logan_ctx* c, int u, const KernelArgs& ka, int phase, cudaStream_t s,
-                const PackedPlan& pk) {
+                const PackedPlan& pk, int units, bool all) {
     cudaError_t e;
-    if (u < kNumLevels && ((pk.levels >> u) & 1u)) {
+    if (u >= kNumLevels && ((pk.levels >> (u - kNumLevels)) & 1u)) {
+        return launch_latency(c, u - kNumLevels, unit_queue(u), units, all, ka, phase, s, pk);
+    } else if (u < kNumLevels && ((pk.levels >> u) & 1u)) {
         const int grid = c->num_sms * std::max(1, c->packed_blocks_per_sm[u]);
-        e = launch_packed_level_persistent(u, ka, pk.args[u], grid, phase, s);
+        e = launch_packed_level(u, ka, pk.args[u], grid, phase, s);
     } else if (u >= kNumLevels) {
         const int l = u - kNumLevels;
         const int grid = c->num_sms * std::max(1, c->twin_blocks_per_sm[l]);
@@ -266,8 +299,10 @@ uint32_t long_item_min(const logan_ctx* c, uint32_t n_items) {
     if (c->long_item == -1) return 0xffffffffu;
     if (c->long_item >= 0) return uint32_t(std::min<int64_t>(c->long_item, 0xfffffffe));
     // automatic: a batch that cannot fill the GPU's warps runs every item in
-    // latency form; otherwise items of 64K bases and more do
-    return n_items <= uint32_t(c->num_sms) * 32u ? 0u : 65536u;
+    // latency form; otherwise items of 128K bases and more do (20,000 uneven
+    // pairs up to 1 Mbp: 226 ms from 64K on, 212 from 128K, 214 from 256K, 249
+    // with none)
+    return n_items <= uint32_t(c->num_sms) * 32u ? 0u : 131072u;
 }
 
 // The auxiliary streams of caller stream `s` (created on first use).
@@ -277,12 +312,12 @@ AuxSet* aux_for(logan_ctx* c, cudaStream_t s) {
     AuxSet a;
     a.main = s;
     bool ok = cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int l = 0; ok && l < kUnits; ++l) {
+    for (int l = 0; ok && l < kStreams; ++l) {
         ok = cudaStreamCreateWithFlags(&a.st[l], cudaStreamNonBlocking) == cudaSuccess &&
              cudaEventCreateWithFlags(&a.join[l], cudaEventDisableTiming) == cudaSuccess;
     }
     if (!ok) {
-        for (int l = 0; l < kUnits; ++l) {
+        for (int l = 0; l < kStreams; ++l) {
             if (a.st[l]) cudaStreamDestroy(a.st[l]);
             if (a.join[l]) cudaEventDestroy(a.join[l]);
         }
@@ -317,6 +352,9 @@ PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int3
         }
         if (packed_plan(sc, xmax, &pk.args[l])) pk.levels |= 1u << l;
     }
+    // levels 0 and 1 run wider windows packed than in 32 bits: their records
+    // need packed readers up to level 2
+    if (!((pk.levels >> 2) & 1u)) pk.levels &= ~3u;
     return pk;
 }
 
@@ -497,6 +535,8 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         if (!(twin_form && tab.long_min == 0u)) start_units |= 1u << l;
         first_escalated = l + 1;
     }
+    const bool all = tab.long_min == 0u;  // every item takes its level's latency form
+    const int units = latency_units(c, n_items, tab.long_min);
     uint32_t p1_levels = 0, p2_levels = 0;
     cudaEvent_t* ev = c->ev;
     auto rec = [&](int idx, cudaStream_t st) {
@@ -524,7 +564,24 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
             cudaStream_t st = ax ? ax->st[u] : s;
             if (ax && cudaStreamWaitEvent(st, ax->fork, 0) != cudaSuccess) return LOGAN_ECUDA;
             if (!rec(EV_P1S + u, st)) return LOGAN_ECUDA;
-            if (launch_unit(c, u, ka, PHASE_INITIAL, st, packed) != LOGAN_OK) return LOGAN_ECUDA;
+            int phase = PHASE_INITIAL;
+            if (u == kTwinLevels && kTwinLevels < kLatencyLevels && ((packed.levels >> u) & 1u) &&
+                tab.long_min != 0xffffffffu) {
+                // the long items of the 512-row level in its latency form, beside the rest
+                cudaStream_t sl = ax ? ax->st[kUnits] : s;
+                if (ax && cudaStreamWaitEvent(sl, ax->fork, 0) != cudaSuccess) return LOGAN_ECUDA;
+                if (launch_latency(c, u, u, 1, all, ka, PHASE_LONG, sl, packed) != LOGAN_OK)
+                    return LOGAN_ECUDA;
+                if (ax && cudaEventRecord(ax->join[kUnits], sl) != cudaSuccess) return LOGAN_ECUDA;
+                phase = PHASE_REST;
+                ++launches;
+            }
+            if (!(phase == PHASE_REST && tab.long_min == 0u) &&
+                launch_unit(c, u, ka, phase, st, packed, units, all) != LOGAN_OK)
+                return LOGAN_ECUDA;
+            if (phase == PHASE_REST && ax &&
+                cudaStreamWaitEvent(st, ax->join[kUnits], 0) != cudaSuccess)
+                return LOGAN_ECUDA;
             if (!rec(EV_P1E + u, st)) return LOGAN_ECUDA;
             if (ax && (cudaEventRecord(ax->join[u], st) != cudaSuccess ||
                        cudaStreamWaitEvent(s, ax->join[u], 0) != cudaSuccess))
@@ -539,7 +596,12 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         for (int u : {lvl, lvl < kTwinLevels && !plain ? kNumLevels + lvl : -1}) {
             if (u < 0) continue;
             if (!rec(EV_P2S + u, s)) return LOGAN_ECUDA;
-            if (launch_unit(c, u, ka, PHASE_ESCALATED, s, packed) != LOGAN_OK) return LOGAN_ECUDA;
+            // (a small batch's bands stay in the latency forms)
+            const bool small = tab.long_min == 0u && u == kTwinLevels && u < kLatencyLevels &&
+                               ((packed.levels >> u) & 1u);
+            if ((small ? launch_latency(c, u, u, 1, all, ka, PHASE_ESCALATED, s, packed)
+                       : launch_unit(c, u, ka, PHASE_ESCALATED, s, packed, units, all)) != LOGAN_OK)
+                return LOGAN_ECUDA;
             if (!rec(EV_P2E + u, s)) return LOGAN_ECUDA;
             p2_levels |= 1u << u;
             ++launches;
@@ -738,6 +800,9 @@ int logan_ctx_create(logan_ctx_t** out, int device, const char* autotune_json) {
         c->blocks_per_sm[l] = l < kWarpLevels ? warp_level_blocks_per_sm(l) : cta_level_blocks_per_sm(l);
     for (int l = 0; l < kNumLevels; ++l)
         c->packed_blocks_per_sm[l] = packed_level(l) ? packed_level_blocks_per_sm(l) : 0;
+    for (int l = 0; l < kLatencyLevels; ++l)
+        for (int k = 0; k < 3; ++k)
+            c->latency_blocks_per_sm[l][k] = packed_latency_blocks_per_sm(l, 1 << k);
     for (int l = 0; l < kTwinLevels; ++l) c->twin_blocks_per_sm[l] = twin_blocks_per_sm(l);
     for (int l = 0; l < affine_levels(); ++l) {
         c->affine_blocks_per_sm[l] = affine_blocks_per_sm(l);
@@ -772,7 +837,7 @@ void logan_ctx_destroy(logan_ctx_t* c) {
     for (auto& ge : c->graphs)
         if (ge.exec) cudaGraphExecDestroy(ge.exec);
     for (auto& a : c->aux) {
-        for (int l = 0; l < kUnits; ++l) {
+        for (int l = 0; l < kStreams; ++l) {
             if (a.st[l]) {
                 cudaStreamSynchronize(a.st[l]);
                 cudaStreamDestroy(a.st[l]);

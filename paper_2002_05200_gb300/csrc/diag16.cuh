@@ -59,36 +59,61 @@ constexpr int kPrefetch = 64;     // steps that the prefetched codes last
 // G lanes of V virtual lanes of 2 R slots
 template <int G, int V, int R>
 struct Diag {
-    static_assert(R == 16 || (R == 8 && V == 1), "registers per virtual lane");
+    static_assert(R == 16 || (V == 1 && (R == 8 || R == 4 || R == 2)), "registers per virtual lane");
     static constexpr int VR = 2 * R;     // slots of a virtual lane
     static constexpr int C = V * VR;     // slots of a lane
     static constexpr int W = G * C;      // slots of the window
-    static constexpr int LOG2W = W == 64    ? 6
+    static constexpr int LOG2W = W == 32    ? 5
+                                 : W == 64  ? 6
                                  : W == 128 ? 7
                                  : W == 256 ? 8
                                  : W == 512 ? 9
                                  : W == 1024 ? 10
                                              : 11;
     static_assert((1 << LOG2W) == W, "window must be a power of two");
+    // anti-diagonals per loop iteration; with two virtual lanes the body of
+    // four costs more in registers than it saves
+    static constexpr int UNROLL = V == 1 ? 4 : 2;
+    // a slide moves the window by half a virtual lane, or by whole lanes (an
+    // eighth of the window) where a virtual lane is short
+    static constexpr int SL = R == 16 ? 0 : (G >= 8 ? G / 8 : 1);
+    static constexpr int SLIDE = R == 16 ? R : SL * VR;
     static constexpr uint32_t VMASK = VR == 32 ? 0xffffffffu : (1u << VR) - 1u;
 };
 
-// Per-unit state, replicated in its lanes.  lo, hi, dn (first row with a
-// column, d - n) and mt (row m) are window slots minus the lane's first slot.
+// Per-unit state, replicated in its lanes except what is marked per lane.
 template <int V>
 struct DState {
-    int lo, hi, dn, mt;
+    int dn, mt;         // first slot with a column and slot of row m, minus the lane's first slot
     int theta;
-    int best, bi, bd;   // bd: anti-diagonal of the best cell
+    int best;
     int X;
     int base, e, phi;
-    uint32_t c32;       // cells since the last fold into `cells`
-    unsigned long long cells, cells0;
+    int bd, br;         // per lane: anti-diagonal and r of the last best cell that this lane found
+    uint32_t c32;       // per lane: cells since the last fold into `cells`
+    unsigned long long cells;   // per lane
+    unsigned long long cells0;  // cells of narrower levels (resumed items), in the leader lane
     uint32_t item;
     bool active, done, overflow, migrated;
+    uint32_t rb[V];                        // slots of the next step's range (without the matrix's bounds)
     uint32_t LE[V], LO[V];                 // live slots on the last even / odd anti-diagonal
     uint32_t a0[V], a1[V], b0[V], b1[V];   // code bit planes, bit k = slot k
     uint32_t na0, na1, nb0, nb1;           // the codes that enter next (a': low bit first, b': high bit first)
+};
+
+// lane masks of a unit of G lanes: the unit's lanes, those below and above
+template <int G>
+struct Lanes {
+    uint32_t all, below, above, prev, next;
+    __device__ __forceinline__ explicit Lanes(int lane) {
+        const int first = lane / G * G;
+        all = G == 32 ? FULL : (((1u << (G & 31)) - 1u) << first);
+        const uint32_t me = 1u << lane;
+        below = all & (me - 1u);
+        above = all & ~(me - 1u) & ~me;
+        prev = (me >> 1) & all;
+        next = (me << 1) & all;
+    }
 };
 
 // 16 two-bit codes (code t at bits 2t) -> their low and high bit planes
@@ -184,21 +209,110 @@ __device__ __forceinline__ uint32_t sign_bytes(uint32_t a, uint32_t b) {
     return r;
 }
 
+// Bit k = sign of slot k's half-word in x[0 .. R).  Four slots' sign bytes per
+// permute; for R >= 8 they are gathered by multiply-adds as 255 * mask (each
+// byte 0 or 255 times its power of two), and 255 * 0xfefefeff = 1 (mod 2^32).
+template <int R>
+__device__ __forceinline__ uint32_t sign_mask(const uint32_t (&x)[R]) {
+    if constexpr (R == 2) {  // bytes: slots 0, 1, 2, 3
+        return ((sign_bytes(x[0], x[1]) & 0x08040201u) * 0x01010101u) >> 24;
+    } else if constexpr (R == 4) {  // byte j: slots 2j and 2j + 1
+        const uint32_t t = (sign_bytes(x[0], x[2]) & 0x40100401u) |
+                           (sign_bytes(x[1], x[3]) & 0x80200802u);
+        return (t * 0x01010101u) >> 24;
+    } else {
+        uint32_t acc = 0u;
+#pragma unroll
+        for (int h = 0; h < R / 2; ++h) acc = sign_bytes(x[h], x[h + R / 2]) * (1u << h) + acc;
+        uint32_t m = acc * 0xfefefeffu;
+        if constexpr (R == 8) {  // byte j: slots 4j .. 4j + 3, nibbles to 16 bits
+            m = m | (m >> 4);
+            m = __byte_perm(m, 0u, 0x4420);
+        }
+        return m;
+    }
+}
+
+// bits from the highest set bit of an N-bit mask downwards (0 for 0)
+template <int N>
+__device__ __forceinline__ uint32_t fill_down(uint32_t m) {
+    if constexpr (N <= 8) {  // shifts and ORs: shorter than a find-leading-one
+        m = m | (m >> 1) | (m >> 2);
+        if constexpr (N == 4) return m | (m >> 3);
+        return m | (m >> 3) | (m >> 6);
+    } else {
+        return __funnelshift_rc(~0u, 0u, __clz(m));
+    }
+}
+
+// The slots of the next anti-diagonal's range [first live, last live + 1] (rows)
+// from the live slots L of this one, without numbers: a slot is in range when
+// a live slot lies at or below its row and one at or above the row before.  ODD: L is
+// of an odd step, the next one (even) sees rows one slot lower.  Returns the
+// warp's vote of lanes with a live slot.
+template <int G, int V, int R, bool ODD>
+__device__ __forceinline__ uint32_t next_range(const uint32_t (&L)[V], const Lanes<G>& ln,
+                                               uint32_t (&rb)[V]) {
+    constexpr int VR = Diag<G, V, R>::VR;
+    uint32_t anyl = L[0];
+    if constexpr (V == 2) anyl |= L[1];
+    const uint32_t vote = __ballot_sync(FULL, anyl != 0u);
+    bool near_;  // the neighbouring lane's slot next to this lane's first (odd: last) one is live
+    if constexpr (G == 1) {
+        near_ = false;
+    } else if constexpr (ODD) {
+        near_ = (__ballot_sync(FULL, (L[0] & 1u) != 0u) & ln.next) != 0u;
+    } else {
+        near_ = (__ballot_sync(FULL, (L[V - 1] >> (VR - 1)) != 0u) & ln.prev) != 0u;
+    }
+    const bool below = (vote & ln.below) != 0u, above = (vote & ln.above) != 0u;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        bool bl = below, ab = above;
+        if constexpr (V == 2) {
+            if (v == 1) bl = bl || L[0] != 0u;
+            else ab = ab || L[1] != 0u;
+        }
+        uint32_t lx, hx;
+        if constexpr (ODD) {
+            // from one slot below the first live one, to the last live one
+            const uint32_t nx = v + 1 < V ? L[v + 1] & 1u : (near_ ? 1u : 0u);
+            lx = (L[v] >> 1) | (L[v] & 1u) | (nx << (VR - 1));
+            hx = L[v];
+        } else {
+            // from the first live slot, to one above the last
+            const uint32_t pv = v > 0 ? L[v - 1] >> (VR - 1) : (near_ ? 1u : 0u);
+            lx = L[v];
+            hx = (L[v] << 1) | pv | (L[v] & (1u << (VR - 1)));
+            if constexpr (VR < 32) hx &= (1u << VR) - 1u;
+        }
+        const uint32_t low = bl ? FULL : (lx | (0u - lx));
+        const uint32_t high = ab ? Diag<G, V, R>::VMASK : fill_down<VR>(hx);
+        rb[v] = low & high;
+    }
+    return vote;
+}
+
 // key of score distance u (>= 0) above a threshold at 32768, slot k of VR
 template <int VR>
 __device__ __forceinline__ uint32_t live_key(int u, int k) {
     return 32768u + uint32_t(u) * uint32_t(KS) + uint32_t(VR - 1 - k);
 }
 
-// Shifts one array's slots by half a virtual lane (R slots): UP moves the
-// window to larger rows (slot s takes what slot s + R held).  Row codes move
-// by +R in the low halves and -R in the high ones.
+// Shifts one array's slots by Diag::SLIDE: UP moves the window to larger rows
+// (slot s takes what slot s + SLIDE held).  By half a virtual lane, row codes
+// move by +R in the low halves and -R in the high ones.
 template <int G, int V, int R, bool UP>
-__device__ __forceinline__ void shift_half(uint32_t (&Q)[V * R], bool on, int gl, uint32_t floor2) {
+__device__ __forceinline__ void shift_slots(uint32_t (&Q)[V * R], bool on, int gl, uint32_t floor2) {
+    constexpr int SL = Diag<G, V, R>::SL;
     constexpr uint32_t rebase = uint32_t(R) - (uint32_t(R) << 16);
 #pragma unroll
     for (int h = 0; h < R; ++h) {
-        if constexpr (UP) {
+        if constexpr (SL > 0) {
+            uint32_t x = UP ? __shfl_down_sync(FULL, Q[h], SL, G) : __shfl_up_sync(FULL, Q[h], SL, G);
+            x = (UP ? gl >= G - SL : gl < SL) ? floor2 : x;
+            Q[h] = on ? x : Q[h];
+        } else if constexpr (UP) {
             uint32_t nx = __shfl_down_sync(FULL, Q[h], 1, G);  // the upper lane's first virtual lane
             nx = gl == G - 1 ? floor2 : nx;
 #pragma unroll
@@ -222,9 +336,14 @@ __device__ __forceinline__ void shift_half(uint32_t (&Q)[V * R], bool on, int gl
 
 // the same for a live mask
 template <int G, int V, int R, bool UP>
-__device__ __forceinline__ void shift_half_mask(uint32_t (&L)[V], bool on, int gl) {
+__device__ __forceinline__ void shift_mask(uint32_t (&L)[V], bool on, int gl) {
+    constexpr int SL = Diag<G, V, R>::SL;
     constexpr uint32_t M = Diag<G, V, R>::VMASK;
-    if constexpr (UP) {
+    if constexpr (SL > 0) {
+        uint32_t x = UP ? __shfl_down_sync(FULL, L[0], SL, G) : __shfl_up_sync(FULL, L[0], SL, G);
+        x = (UP ? gl >= G - SL : gl < SL) ? 0u : x;
+        L[0] = on ? x : L[0];
+    } else if constexpr (UP) {
         uint32_t nx = __shfl_down_sync(FULL, L[0], 1, G);
         nx = gl == G - 1 ? 0u : nx;
 #pragma unroll

@@ -71,8 +71,9 @@ struct DiagArgs {
     int mp;      // max(match, 0)
     int step;    // theta's growth per anti-diagonal: 32 * -gap
     int floor;   // smallest key (a dead one)
-    int iters;   // loop iterations (two anti-diagonals each) between renormalisations
-    int unit;    // match - mismatch == 2 * (mismatch - 2 gap): one multiply-add per substitution
+    int period;  // anti-diagonals between renormalisations (a power of two, 4 .. 64)
+    int unit;    // match 1 and match - mismatch == 2 * (mismatch - 2 gap) (as +1/-1/-1): one
+                 // multiply-add per substitution, a best that grows by 1 at most per anti-diagonal
     // multipliers of a mask bit at position p: mismatch - 2 gap and match -
     // mismatch in key units, divided by 2^p
     uint32_t cb[6], cf[6];
@@ -88,9 +89,15 @@ int warp_level_blocks_per_sm(int level);
 bool packed_level(int level);
 // the constants for this scoring and X, false when the scores do not fit
 bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da);
-cudaError_t launch_packed_level_persistent(int level, const KernelArgs& ka, const DiagArgs& da,
-                                           int grid, int phase, cudaStream_t s);
+cudaError_t launch_packed_level(int level, const KernelArgs& ka, const DiagArgs& da, int grid,
+                                int phase, cudaStream_t s);
 int packed_level_blocks_per_sm(int level);
+// latency forms of levels 0-4 (windows of 128, 128, 128, 256, 512 rows): 1, 2
+// or 4 extensions per warp in short lanes
+constexpr int kLatencyLevels = 5;
+cudaError_t launch_packed_latency(int level, int queue, int units, const KernelArgs& ka,
+                                  const DiagArgs& da, int grid, int phase, cudaStream_t s);
+int packed_latency_blocks_per_sm(int level, int units);
 // level k's one-warp form (k < kTwinLevels), persistent over twin_queue(k)
 cudaError_t launch_twin_persistent(int level, const KernelArgs& ka, int grid, int phase,
                                    cudaStream_t s);

@@ -83,7 +83,8 @@ __host__ __device__ constexpr int level_window(int k) { return level_cells(k) * 
 // which keeps the lanes busy but makes every anti-diagonal step of one
 // extension cost a whole warp's instructions.  A long item (the one a
 // batch waits for) or an item of a batch too small to fill the GPU runs
-// instead in its level's latency form: the same window, one warp of 32
+// instead in its level's latency form.  Packed levels have their own
+// (xdrop_diag16.cu); the 32-bit one is the same window on one warp of 32
 // lanes x window/32 rows, so a step is about half the instructions and its
 // reductions are single warp reductions.  (A 4-warp block form of the
 // 512-row level, one barrier per step, measured 2x slower per step than
@@ -104,6 +105,8 @@ struct Counters {
     unsigned long long cells[kNumLevels + 1];  // cells computed by each level (both forms)
     unsigned int mig_used[kNumLevels];         // migration records written per level
     unsigned int head2[kQueues];               // pop cursor of the escalated entries
+    unsigned int n_long[kNumLevels];           // binned entries for the latency form (the first ones)
+    unsigned int head_long[kNumLevels];        // their pop cursor
 };
 
 // Which entries of a level's queue a launch processes: the binned (initial)
@@ -113,28 +116,39 @@ constexpr int PHASE_INITIAL = 0;
 constexpr int PHASE_ESCALATED = 1;
 constexpr int PHASE_PLAIN = 2;
 constexpr int PHASE_WHOLE = 3;  // every entry [0, tail): levels that run one after another
+constexpr int PHASE_LONG = 4;   // the binned entries [0, n_long): a level's latency form
+constexpr int PHASE_REST = 5;   // the other binned entries, [n_long, started)
 
 // Queue slot of each idle unit of a warp (the units whose leader lane is set
 // in `want`; `unit` is this lane's unit of G lanes).  A warp's first call in
-// a launch takes static slots -- unit u of the launch's warp w gets entry
-// w * (32 / G) + u of the phase's range -- so the first entries (the
-// longest: binning orders a queue longest first) go to the warps in launch
-// order, and with them to the SMs and their schedulers in turn (a block's
-// warps sit on one SM's four schedulers, consecutive blocks on different
-// SMs), instead of following the order in which warps reach an atomic;
-// consecutive entries share a warp, so its units start on items of similar
-// length.  Later calls pop dynamically after the static entries.  Every
-// unit must be idle at the first call (true at kernel start).  Returns the
-// slot; one at or past `limit` means the range is used up.
+// a launch takes static slots -- unit u of the launch's warp w gets
+// entry w * (32 / G) + u of the phase's range.  Binning orders a queue longest
+// first, so consecutive entries, of similar length, share a warp, and a block's
+// warps; block b takes rank perm(b), which spreads the lengths over the SMs
+// whichever way the blocks reach them: in turn (an SM holds blocks s, s + SMs,
+// ...: one of each quarter) or, when another launch's blocks leave an SM's
+// slots at once, four consecutive ones (also one of each quarter; in block
+// order, 20,000 extensions took 7.4-7.9 ms beside an empty launch and 5.8 ms
+// alone).  Later calls pop dynamically after the static entries.  Every unit
+// must be idle at the first call (true at kernel start).
+// Returns the slot; one at or past `limit` means the range is used up.
 template <int G>
 __device__ __forceinline__ unsigned int pop_unit_slot(Counters* c, int q, int phase, uint32_t want,
                                                       int lane, int unit, bool& first_wave,
                                                       unsigned int& limit) {
     constexpr unsigned int U = 32 / G;
     const unsigned int nwarps = gridDim.x * (blockDim.x >> 5);
-    const unsigned int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const unsigned int lo = phase == PHASE_ESCALATED ? c->started[q] : 0u;
-    limit = phase == PHASE_INITIAL ? c->started[q] : c->tail[q];
+    // perm: block k * q + r (k < 4, r < q) -> ((r + k) mod 4) * q + r
+    const unsigned int q4 = gridDim.x >> 2, b = blockIdx.x;
+    const unsigned int k = q4 ? b / q4 : 4u, r = b - k * q4;
+    const unsigned int rank = k < 4u ? ((r + k) & 3u) * q4 + r : b;
+    const unsigned int gw = rank * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const unsigned int lo = phase == PHASE_ESCALATED ? c->started[q]
+                            : phase == PHASE_REST    ? c->n_long[q]
+                                                     : 0u;
+    limit = phase == PHASE_INITIAL || phase == PHASE_REST ? c->started[q]
+            : phase == PHASE_LONG                         ? c->n_long[q]
+                                                          : c->tail[q];
     if (first_wave) {
         first_wave = false;
         return lo + gw * U + unsigned(unit);
@@ -142,7 +156,9 @@ __device__ __forceinline__ unsigned int pop_unit_slot(Counters* c, int q, int ph
     const int leader = __ffs(want) - 1;
     unsigned int first = 0u;
     if (lane == leader)
-        first = atomicAdd(phase == PHASE_ESCALATED ? &c->head2[q] : &c->head[q],
+        first = atomicAdd(phase == PHASE_ESCALATED ? &c->head2[q]
+                          : phase == PHASE_LONG    ? &c->head_long[q]
+                                                   : &c->head[q],
                           unsigned(__popc(want)));
     first = __shfl_sync(0xffffffffu, first, leader);
     return lo + U * nwarps + first + unsigned(__popc(want & ((1u << (unit * G)) - 1u)));
@@ -172,7 +188,11 @@ enum MigField {
 };
 constexpr int MIG_RELATIVE = 1;
 constexpr int MIG_ABSOLUTE = 2;
-__host__ __device__ constexpr int mig_stride(int level) { return kMigHeader + 2 * level_window(level); }
+// rows of a level's record: its packed forms may hold a wider window
+__host__ __device__ constexpr int mig_rows(int level) {
+    return level_window(level) < 128 ? 128 : level_window(level);
+}
+__host__ __device__ constexpr int mig_stride(int level) { return kMigHeader + 2 * mig_rows(level); }
 
 // One 2-bit code of a pool (p must lie inside the pool).
 __device__ __forceinline__ uint32_t code_at(const uint32_t* __restrict__ w, int64_t p) {

@@ -168,9 +168,14 @@ __global__ void k_bin_hist(const Item* __restrict__ items, uint32_t n, LevelTabl
 // one block of kBuckets threads: per queue exclusive scan of the bucket
 // counts (longest bucket first) -> cursors; queue sizes -> counters (the
 // fallback ring's queue gets no binned items)
-__global__ void k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c) {
+__global__ void k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c,
+                           uint32_t long_min) {
     __shared__ uint32_t s[kBuckets];
     const int t = threadIdx.x;
+    // buckets that hold only items of m + n >= long_min come first
+    const int n_long_buckets = long_min == 0u            ? kBuckets
+                               : long_min == 0xffffffffu ? 0
+                                                         : kBuckets - 1 - work_bucket(long_min - 1u, 0u);
     for (int l = 0; l < kQueues; ++l) {
         const uint32_t v = hist[l * kBuckets + t];
         s[t] = v;
@@ -186,6 +191,7 @@ __global__ void k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c
             c->tail[l] = s[t];
             c->started[l] = s[t];
         }
+        if (l < kNumLevels && t == 0) c->n_long[l] = n_long_buckets ? s[n_long_buckets - 1] : 0u;
         __syncthreads();
     }
     if (t < kQueues) {
@@ -193,7 +199,10 @@ __global__ void k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c
         c->head2[t] = 0u;
     }
     if (t <= kNumLevels) c->cells[t] = 0ull;
-    if (t < kNumLevels) c->mig_used[t] = 0u;
+    if (t < kNumLevels) {
+        c->mig_used[t] = 0u;
+        c->head_long[t] = 0u;
+    }
 }
 
 __global__ void k_bin_scatter(const Item* __restrict__ items, uint32_t n, LevelTable table,
@@ -219,7 +228,11 @@ __global__ void k_reset_counters(Counters* c, uint32_t first_items, int first_le
     if (t <= kNumLevels) c->cells[t] = 0ull;
     (void)first_items;
     (void)first_level;
-    if (t < kNumLevels) c->mig_used[t] = 0u;
+    if (t < kNumLevels) {
+        c->mig_used[t] = 0u;
+        c->n_long[t] = 0u;
+        c->head_long[t] = 0u;
+    }
 }
 
 struct ResultOut {
@@ -293,7 +306,7 @@ cudaError_t launch_bin(const Item* items, uint32_t n_items, LevelTable table, in
         const unsigned int g = min(blocks_for(n_items, 256), 1024u);
         k_bin_hist<<<g, 256, 0, s>>>(items, n_items, table, force_level, maxl, hist);
     }
-    k_bin_scan<<<1, kBuckets, 0, s>>>(hist, counters);
+    k_bin_scan<<<1, kBuckets, 0, s>>>(hist, counters, table.long_min);
     if (n_items)
         k_bin_scatter<<<blocks_for(n_items, 256), 256, 0, s>>>(items, n_items, table, force_level,
                                                                maxl, hist, queues, qcap);

@@ -285,10 +285,12 @@ int launch(logan_server* s, uint64_t ticket, Req& q) {
     if (e == cudaSuccess) e = h2d(seeds, r.seeds, size_t(r.n_pairs) * sizeof(logan_seed_t));
     if (e == cudaSuccess && xs) e = h2d(xs, r.X_per_pair, size_t(r.n_pairs) * 4);
     if (e != cudaSuccess) return LOGAN_ECUDA;
-    // with the GPU nearly idle, long extensions run one to a warp (shorter
-    // latency); with several requests in flight every extension runs in the
-    // several-to-a-warp forms (more extensions per instruction)
-    logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, s->running.load() <= 8 ? 65536 : -1);
+    // long extensions run one to a warp (the step that a request's latency
+    // waits for); with many requests in flight only the longest ones do (more
+    // extensions per instruction for the rest).  A burst of 24 requests of up
+    // to 1,000 uneven pairs: 192 ms with none, 147 ms from 200,000 bases on,
+    // 128 ms from 65,536 on
+    logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, s->running.load() <= 8 ? 65536 : 131072);
     int rc = logan_extend_batch(s->ctx, &dA, &dB, reinterpret_cast<const logan_seed_t*>(seeds),
                                 r.n_pairs, r.match, r.mismatch, r.gap, r.X,
                                 reinterpret_cast<const int32_t*>(xs), ws, q.ws_bytes,

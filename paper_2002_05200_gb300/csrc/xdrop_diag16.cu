@@ -17,31 +17,27 @@
 // Then every half-word stays inside [0, 65536) through every addition, and an
 // addition of both halves is one 32-bit operation.
 //
-// Bound by the ALU pipe and issue together (about 7.5 instructions per pair
-// of cells, 3 of them on the ALU pipe, and about 100 of bookkeeping per lane
-// and anti-diagonal).  The row-window form it replaced (a prune select, range
-// test and re-basing per cell, three rotating arrays, a slide of the window
-// every 16 rows) ran 12 per pair of cells and about 140 of bookkeeping.
-// 100,000 lognormal pairs, X = 100: level 2 (137e9 cells) 83 -> 52 ms, level 5
-// (105e9) 52 -> 44 ms, level 6 19.5 -> 9 ms, the whole call 182 -> 123 ms.
+// Bound by the ALU pipe and issue together: about 7 instructions per pair of
+// cells and 90 of bookkeeping per lane and anti-diagonal (level 2: 206 per
+// warp and anti-diagonal, 79 % of issue slots, ALU pipe 79 %).  The
+// bookkeeping has no numbers to reduce: ranges pass between anti-diagonals as
+// masks and two votes, the best as one vote and a note in the lane that has
+// it, cells as population counts, all summed when the extension ends.
+// 100,000 lognormal pairs, X = 100: level 2 (137e9 cells) 83 ms in the
+// row-window form this replaced, 52 with lo / hi / best reduced by shuffles,
+// 47 now; level 5 (105e9) 52, 44, 41; the whole call 182, 123, 113 ms.
+//
+// Latency forms: a lone extension waits for its own chain, so short lanes
+// (4 to 16 slots) cut the instructions per anti-diagonal: 112 with 4 slots per
+// lane, 140 ns per anti-diagonal on an idle SM (175 ns in the 32-bit one-warp
+// form).
+#include <algorithm>
+
 #include "diag16.cuh"
 
 namespace logan {
 
 namespace {
-
-constexpr int kGone = 1 << 20;  // `lo` of a unit without a range
-
-// lo, hi, dn and mt of rows / diagonals given in window coordinates
-template <int G, int V, int R>
-__device__ __forceinline__ void set_range(DState<V>& u, const Item& it, int lo_row, int hi_row,
-                                          int gl) {
-    const int off = u.base + u.e + gl * Diag<G, V, R>::C;
-    u.lo = lo_row - off;
-    u.hi = hi_row - off;
-    u.dn = 2 * u.e + 1 - u.phi - int(it.n) - off;
-    u.mt = int(it.m) - off;
-}
 
 template <int G, int V, int R>
 __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
@@ -53,6 +49,7 @@ __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs&
     u.X = it.X;
     u.c32 = 0u;
     u.theta = 32768;
+    bool fits = true;
     const int32_t slot = ka.mig_slot[id];
     const int32_t* rec = slot >= 0 ? mig_record(ka, slot) : nullptr;
     if (rec && rec[MIG_KIND] == MIG_RELATIVE) {
@@ -63,10 +60,10 @@ __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs&
         u.e = (d + u.phi - 1) >> 1;
         u.base = ((lo + hi) >> 1) - u.e - D::W / 2;
         u.best = rec[MIG_BEST];
-        u.bi = rec[MIG_BI];
         u.bd = rec[MIG_BI] + rec[MIG_BJ];
-        u.cells = (unsigned long long)uint32_t(rec[MIG_CELLS_LO]) |
-                  ((unsigned long long)uint32_t(rec[MIG_CELLS_HI]) << 32);
+        u.br = rec[MIG_BI] - ((u.bd + u.phi) >> 1);
+        u.cells0 = (unsigned long long)uint32_t(rec[MIG_CELLS_LO]) |
+                   ((unsigned long long)uint32_t(rec[MIG_CELLS_HI]) << 32);
         // d-1 (even) relative to T1, d-2 (odd) relative to T2, onto theta = 32768
         const int c1 = rec[MIG_T1] - rec[MIG_T] + da.gap;
         const int c2 = rec[MIG_T2] - rec[MIG_T] + 2 * da.gap;
@@ -94,56 +91,80 @@ __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs&
             u.LE[v] = le;
             u.LO[v] = lo_;
         }
-        set_range<G, V, R>(u, it, lo, hi, gl);
+        // a record as wide as this window (levels whose forms share one) stays
+        // as it is for the next level
+        const int first = u.base + u.e;
+        fits = lo - first >= D::UNROLL / 2 && hi - first < D::W - D::UNROLL / 2;
     } else {
         // S(0,0) = 0 on d = 0 (even), X above its threshold, mid-window
         u.phi = 0;
         u.e = 0;
         u.base = -D::W / 2;
-        u.best = u.bi = u.bd = 0;
-        u.cells = 0ull;
+        u.best = u.bd = u.br = 0;
+        u.cells0 = 0ull;
         const uint32_t f2 = uint32_t(da.floor) * 0x10001u;
 #pragma unroll
         for (int h = 0; h < V * R; ++h) QE[h] = QO[h] = f2;
 #pragma unroll
         for (int v = 0; v < V; ++v) u.LE[v] = u.LO[v] = 0u;
-        if (gl == G / 2) {  // slot W / 2 is the first of this lane (G = 1: of virtual lane V / 2)
-            constexpr int v0 = G == 1 ? V / 2 : 0;
-            QE[v0 * R] = (f2 & 0xffff0000u) | live_key<D::VR>(it.X, 0);
-            u.LE[v0] = 1u;
+        if (gl == G / 2) {  // slot W / 2 is the first of this lane
+            static_assert(G > 1, "lanes");
+            QE[0] = (f2 & 0xffff0000u) | live_key<D::VR>(it.X, 0);
+            u.LE[0] = 1u;
         }
         u.theta += KS * -da.gap;  // theta_1
-        set_range<G, V, R>(u, it, 0, 0, gl);
     }
-    u.cells0 = u.cells;
+    u.cells = 0ull;
+    const int off = u.base + u.e + gl * D::C;
+    u.dn = 2 * u.e + 1 - u.phi - int(it.n) - off;
+    u.mt = int(it.m) - off;
     load_planes<G, V, R>(ka, it, u, gl);
-    u.active = true;
-    u.done = false;
-    u.overflow = false;
+    u.active = fits;
+    u.done = !fits;
+    u.overflow = !fits;
     u.migrated = false;
 }
 
-// Result or escalation of a finished unit (its leader lane writes).
-template <int V>
-__device__ __forceinline__ void unit_end(const KernelArgs& ka, DState<V>& u, int level, int gl,
-                                         bool twin) {
-    u.cells += u.c32;
-    u.c32 = 0u;
-    if (gl != 0) return;
+// The unit's last best cell (its lanes' latest) and the cells of this level.
+template <int G, int V>
+__device__ __forceinline__ void unit_totals(const DState<V>& u, int& bd, int& br,
+                                            unsigned long long& cells) {
+    bd = u.bd;
+    br = u.br;
+    cells = u.cells + u.c32;
+#pragma unroll
+    for (int o = G / 2; o >= 1; o >>= 1) {
+        const int d = __shfl_xor_sync(FULL, bd, o, G), r = __shfl_xor_sync(FULL, br, o, G);
+        cells += __shfl_xor_sync(FULL, cells, o, G);
+        if (d > bd) {  // (equal ones are copies of the cell the unit started with)
+            bd = d;
+            br = r;
+        }
+    }
+}
+
+// Result or escalation of the finished units (their leader lanes write).
+template <int G, int V>
+__device__ __forceinline__ void units_end(const KernelArgs& ka, DState<V>& u, int level, int gl,
+                                          bool twin) {
+    int bd, br;
+    unsigned long long cells;
+    unit_totals<G, V>(u, bd, br, cells);
+    if (!u.done || gl != 0) return;
     if (u.overflow) {
-        if (u.migrated) atomicAdd(&ka.counters->cells[level], u.cells - u.cells0);
+        if (u.migrated) atomicAdd(&ka.counters->cells[level], cells);
         const int nq = escalate_queue(ka, level, twin);
         const unsigned int t = atomicAdd(&ka.counters->tail[nq], 1u);
         ka.queues[size_t(nq) * ka.qcap + t] = u.item;
     } else {
         ExtRes r;
         r.best = u.best;
-        r.bi = u.bi;
-        r.bj = u.bd - u.bi;
+        r.bi = br + ((bd + u.phi) >> 1);
+        r.bj = bd - r.bi;
         r.status = 0;
-        r.cells = u.cells;
+        r.cells = u.cells0 + cells;
         ka.ext[u.item] = r;
-        atomicAdd(&ka.counters->cells[level], u.cells - u.cells0);
+        atomicAdd(&ka.counters->cells[level], cells);
     }
 }
 
@@ -152,7 +173,8 @@ __device__ __forceinline__ void unit_end(const KernelArgs& ka, DState<V>& u, int
 // which no live cell of d-2 or d-1 lies below.
 template <int G, int V, int R>
 __device__ __forceinline__ void save_band(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
-                                          int32_t slot, int level, int gl,
+                                          int32_t slot, int level, int gl, int lo, int hi, int bd,
+                                          int br, unsigned long long cells,
                                           const uint32_t (&QE)[V * R], const uint32_t (&QO)[V * R]) {
     using D = Diag<G, V, R>;
     int32_t* rec = mig_record(ka, slot);
@@ -187,15 +209,16 @@ __device__ __forceinline__ void save_band(const KernelArgs& ka, const DiagArgs& 
         rec[MIG_ROWS] = rows;
         rec[MIG_D] = 2 * u.e + 1 - u.phi;
         rec[MIG_BASE] = row0;
-        rec[MIG_LO] = u.lo + off;
-        rec[MIG_HI] = u.hi + off;
+        rec[MIG_LO] = lo + off;
+        rec[MIG_HI] = hi + off;
         rec[MIG_BEST] = u.best;
         rec[MIG_T] = T;
         rec[MIG_T1] = T - ref;
         rec[MIG_T2] = T - ref;
-        rec[MIG_BI] = u.bi;
-        rec[MIG_BJ] = u.bd - u.bi;
-        const unsigned long long c = u.cells + u.c32;
+        const int bi = br + ((bd + u.phi) >> 1);
+        rec[MIG_BI] = bi;
+        rec[MIG_BJ] = bd - bi;
+        const unsigned long long c = u.cells0 + cells;
         rec[MIG_CELLS_LO] = int32_t(uint32_t(c));
         rec[MIG_CELLS_HI] = int32_t(uint32_t(c >> 32));
         rec[MIG_LEVEL] = level;
@@ -203,44 +226,49 @@ __device__ __forceinline__ void save_band(const KernelArgs& ka, const DiagArgs& 
     }
 }
 
-// Loop top, before an odd step: units whose range ended are done; windows
-// whose band comes within a slot of an edge slide by half virtual lanes, or
-// overflow when the band does not fit.
+// Loop top, before an odd step, when some unit's band touches its window's
+// outermost slots (every two steps reach one slot further): the window slides by half a virtual lane, or overflows when the band does
+// not fit.
 template <int G, int V, int R>
-__device__ __forceinline__ void unit_prepare(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
-                                             int level, int gl, int unit, uint32_t (&QE)[V * R],
-                                             uint32_t (&QO)[V * R]) {
+__device__ __forceinline__ void units_slide(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
+                                            int level, int gl, int unit, const Lanes<G>& ln,
+                                            uint32_t brink_top, uint32_t brink_bot,
+                                            uint32_t (&QE)[V * R], uint32_t (&QO)[V * R]) {
     using D = Diag<G, V, R>;
-    if (u.active && u.lo >= kGone / 2) {
-        u.active = false;
-        u.done = true;
-    }
-    // the next two steps reach slots lo - 1 .. hi + 1 (of rows inside the matrix)
-    const int off = gl * D::C;
-    const int lo_s = max(u.lo, u.dn) + off, hi_s = min(u.hi, u.mt) + off;
-    bool up = u.active && hi_s > D::W - 2, dn = u.active && lo_s < 1;
-    if (!__any_sync(FULL, up || dn)) return;
+    constexpr int VR = D::VR;
     const uint32_t f2 = uint32_t(da.floor) * 0x10001u;
-    const bool ovf = (up && lo_s - R < 1) || (dn && hi_s + R > D::W - 2);
-    up = up && !ovf;
-    dn = dn && !ovf;
+    const uint32_t Lf = u.LE[0], Ll = u.LE[V - 1];
+    const bool at_top = (__ballot_sync(FULL, (Ll & brink_top) != 0u) & ln.all) != 0u;
+    const bool at_bot = (__ballot_sync(FULL, (Lf & brink_bot) != 0u) & ln.all) != 0u;
+    // live slots that the shifted window would lose or have on its brink
+    uint32_t low, high;
+    constexpr uint32_t bot = (1u << (D::UNROLL / 2)) - 1u, top = bot << (VR - D::UNROLL / 2);
+    if constexpr (D::SL > 0) {
+        low = gl < D::SL ? D::VMASK : gl == D::SL ? bot : 0u;
+        high = gl >= G - D::SL ? D::VMASK : gl == G - D::SL - 1 ? top : 0u;
+    } else {
+        low = brink_bot ? (bot << R) | ((1u << R) - 1u) : 0u;
+        high = brink_top ? (top >> R) | (((1u << R) - 1u) << R) : 0u;
+    }
+    const bool in_low = (__ballot_sync(FULL, (Lf & low) != 0u) & ln.all) != 0u;
+    const bool in_high = (__ballot_sync(FULL, (Ll & high) != 0u) & ln.all) != 0u;
+    const bool ovf = u.active && ((at_top && in_low) || (at_bot && in_high));
+    const bool up = u.active && at_top && !ovf, dn = u.active && at_bot && !ovf;
     if (__any_sync(FULL, up)) {
-        shift_half<G, V, R, true>(QE, up, gl, f2);
-        shift_half<G, V, R, true>(QO, up, gl, f2);
-        shift_half_mask<G, V, R, true>(u.LE, up, gl);
-        shift_half_mask<G, V, R, true>(u.LO, up, gl);
+        shift_slots<G, V, R, true>(QE, up, gl, f2);
+        shift_slots<G, V, R, true>(QO, up, gl, f2);
+        shift_mask<G, V, R, true>(u.LE, up, gl);
+        shift_mask<G, V, R, true>(u.LO, up, gl);
     }
     if (__any_sync(FULL, dn)) {
-        shift_half<G, V, R, false>(QE, dn, gl, f2);
-        shift_half<G, V, R, false>(QO, dn, gl, f2);
-        shift_half_mask<G, V, R, false>(u.LE, dn, gl);
-        shift_half_mask<G, V, R, false>(u.LO, dn, gl);
+        shift_slots<G, V, R, false>(QE, dn, gl, f2);
+        shift_slots<G, V, R, false>(QO, dn, gl, f2);
+        shift_mask<G, V, R, false>(u.LE, dn, gl);
+        shift_mask<G, V, R, false>(u.LO, dn, gl);
     }
     if (up || dn) {
-        const int by = up ? R : -R;
+        const int by = up ? D::SLIDE : -D::SLIDE;
         u.base += by;
-        u.lo -= by;
-        u.hi -= by;
         u.dn -= by;
         u.mt -= by;
         load_planes<G, V, R>(ka, ka.items[u.item], u, gl);
@@ -249,13 +277,30 @@ __device__ __forceinline__ void unit_prepare(const KernelArgs& ka, const DiagArg
         int32_t slot = -1;
         if (ovf && gl == 0) slot = mig_alloc(ka, level);
         slot = __shfl_sync(FULL, slot, unit * G);
+        // first and last live slots, the best cell, the cells
+        int lo = D::W, hi = -1, bd, br;
+        unsigned long long cells;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            if (u.LE[v]) {
+                lo = min(lo, gl * D::C + v * VR + __ffs(u.LE[v]) - 1);
+                hi = gl * D::C + v * VR + 31 - __clz(u.LE[v]);
+            }
+#pragma unroll
+        for (int o = G / 2; o >= 1; o >>= 1) {
+            lo = min(lo, __shfl_xor_sync(FULL, lo, o, G));
+            hi = max(hi, __shfl_xor_sync(FULL, hi, o, G));
+        }
+        unit_totals<G, V>(u, bd, br, cells);
         if (ovf) {
-            if (slot >= 0) save_band<G, V, R>(ka, da, u, slot, level, gl, QE, QO);
+            if (slot >= 0)
+                save_band<G, V, R>(ka, da, u, slot, level, gl, lo, hi, bd, br, cells, QE, QO);
             u.active = false;
             u.done = true;
             u.overflow = true;
             u.migrated = slot >= 0;
-            u.lo = kGone;
+#pragma unroll
+            for (int v = 0; v < V; ++v) u.LE[v] = u.LO[v] = 0u;
         }
     }
 }
@@ -281,13 +326,14 @@ __device__ __forceinline__ void unit_maintain(const KernelArgs& ka, const DiagAr
 }
 
 // One anti-diagonal of every unit of the warp: Q (d-2 on entry) receives d,
-// P holds d-1.  Units without a range compute values without effects.
+// P holds d-1; inm: the lane's slots inside the matrix.  Returns the warp's vote of lanes with a live slot.  Units without a
+// range compute values without effects.
 template <int G, int V, int R, bool UNIT, bool ODD>
-__device__ __forceinline__ void dstep(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
-                                      int gl, uint32_t (&Q)[V * R], const uint32_t (&P)[V * R]) {
+__device__ __forceinline__ uint32_t dstep(const DiagArgs& da, DState<V>& u, int at, int gl,
+                                          const Lanes<G>& ln, const uint32_t (&inm)[V],
+                                          uint32_t (&Q)[V * R], const uint32_t (&P)[V * R]) {
     using D = Diag<G, V, R>;
-    constexpr int VR = D::VR, C = D::C, W = D::W;
-    const int rlo = max(u.lo, u.dn), rhi = min(u.hi + 1, u.mt);
+    constexpr int VR = D::VR, C = D::C;
     // the moving operand's codes
     if constexpr (ODD) {
 #pragma unroll
@@ -324,21 +370,26 @@ __device__ __forceinline__ void dstep(const KernelArgs& ka, const DiagArgs& da, 
     }
     // v >= theta  <=>  bit 15 of v + (32768 - theta)
     const uint32_t thr = uint32_t(32768 - u.theta) * 0x10001u;
-    uint32_t fkey = 0u;
+    uint32_t key = 0u;  // the lane's largest key and its slot in the lane
+    int key_slot = 0;
     uint32_t L[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        // slots of this virtual lane inside [rlo, rhi], then those whose
-        // diagonal predecessor is live (rm), then the matches among them (fm)
-        const int k0 = __viaddmin_s32_relu(rlo, -v * VR, VR);
-        const int k1 = __viaddmin_s32_relu(rhi, 1 - v * VR, VR);
-        const uint32_t s0 = __funnelshift_lc(~0u, 0u, k0), s1 = __funnelshift_lc(~0u, 0u, k1);
-        uint32_t rm = s1 & ~s0 & (ODD ? u.LO[v] : u.LE[v]);
+        // slots in range, then those whose diagonal predecessor is live (rm),
+        // then the matches among them (fm)
+        const uint32_t rb = u.rb[v] & inm[v];
+        u.c32 += uint32_t(__popc(rb));
+        uint32_t rm = rb & (ODD ? u.LO[v] : u.LE[v]);
         uint32_t fm = rm & ~(u.a0[v] ^ u.b0[v]);
         fm = fm & ~(u.a1[v] ^ u.b1[v]);
-        if constexpr (R == 8) {  // slots 8..15 to the upper half-word
+        // slot h + R of register h to bit h + 16 (for R < 8 the bits between
+        // hold copies that no register's mask picks)
+        if constexpr (R == 8) {
             rm = __byte_perm(rm, 0u, 0x4140);
             fm = __byte_perm(fm, 0u, 0x4140);
+        } else if constexpr (R < 8) {
+            rm *= 1u + (1u << (16 - R));
+            fm *= 1u + (1u << (16 - R));
         }
         uint32_t wa, wb;
         if constexpr (UNIT) {
@@ -390,72 +441,41 @@ __device__ __forceinline__ void dstep(const KernelArgs& ka, const DiagArgs& da, 
             x[h] = val + thr;
             if (h & 1) lk = __vimax3_u16x2(lk, Q[g - 1], val);
         }
-        // the signs of four slots per byte permute, gathered as 255 * mask
-        uint32_t acc = 0u;
-#pragma unroll
-        for (int h = 0; h < R / 2; ++h) acc = sign_bytes(x[h], x[h + R / 2]) * (1u << h) + acc;
-        uint32_t m = acc * 0xfefefeffu;  // 255 * 0xfefefeff = 1 (mod 2^32)
-        if constexpr (R == 8) {          // nibbles in bytes -> 16 bits
-            m = m | (m >> 4);
-            m = __byte_perm(m, 0u, 0x4420);
-        }
-        L[v] = m & s1 & ~s0;
-        // the virtual lane's best key, widened with its position
+        L[v] = sign_mask<R>(x) & rb;
         const uint32_t lkey = max(lk & 0xffffu, lk >> 16);
-        const int above = int(lkey) - u.theta;
-        const uint32_t fk = above >= 0 ? ((uint32_t(above) >> LOG2KS) << D::LOG2W) +
-                                             (uint32_t(W - VR - v * VR - gl * C) + (lkey & uint32_t(VR - 1)))
-                                       : 0u;
-        fkey = max(fkey, fk);
-    }
-    // the lane's first / last live slots, then the unit's
-    int fr, lr;
-    bool any;
-    if constexpr (V == 1) {
-        fr = __ffs(L[0]) - 1;
-        lr = 31 - __clz(L[0]);
-        any = L[0] != 0u;
-    } else {
-        const unsigned long long LL = (unsigned long long)L[0] | ((unsigned long long)L[1] << 32);
-        fr = __ffsll(LL) - 1;
-        lr = 63 - __clzll(LL);
-        any = LL != 0ull;
+        // (equal scores: the lower virtual lane's rows come first)
+        const bool more = v == 0 || (lkey >> LOG2KS) > (key >> LOG2KS);
+        key = more ? lkey : key;
+        key_slot = more ? v * VR + VR - 1 - int(lkey & uint32_t(VR - 1)) : key_slot;
     }
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         if constexpr (ODD) u.LO[v] = L[v];
         else u.LE[v] = L[v];
     }
-    const uint32_t flw =
-        any ? (uint32_t(W - gl * C - fr) | (uint32_t(gl * C + 1 + lr) << 16)) : 0u;
-    const uint32_t wkey = unit_max_u32<G>(fkey);
-    uint32_t fl;
-    if constexpr (G == 32) {
-        const uint32_t vote = __ballot_sync(FULL, any);
-        const uint32_t f = __shfl_sync(FULL, flw, __ffs(vote) - 1);
-        const uint32_t l = __shfl_sync(FULL, flw, 31 - __clz(vote));
-        fl = vote ? __byte_perm(f, l, 0x7610) : 0u;
+    // a new best (S > best <=> S - T_d > X) and the first lane that has it;
+    // slots outside the range never hold one
+    int gain;
+    bool mine;
+    if constexpr (UNIT) {  // one match scores 1, so the best grows by 1 at most
+        const bool hit = int(key) >= u.theta + KS * (u.X + 1);
+        const uint32_t vote = __ballot_sync(FULL, hit);
+        gain = (vote & ln.all) != 0u ? 1 : 0;
+        mine = hit && (vote & ln.below) == 0u;
     } else {
-        fl = unit_max_u16x2<G>(flw);
+        const int above = int(key) - u.theta;
+        const uint32_t mine_u = above >= 0 ? uint32_t(above) >> LOG2KS : 0u;
+        const uint32_t top = unit_max_u32<G>(mine_u);
+        gain = max(int(top) - u.X, 0);
+        const bool hit = gain > 0 && mine_u == top;
+        const uint32_t vote = __ballot_sync(FULL, hit);
+        mine = hit && (vote & ln.below) == 0u;
     }
-    const bool run = rlo <= rhi;
-    u.c32 += run ? uint32_t(rhi - rlo + 1) : 0u;
-    // the anti-diagonal's outcome: it advances when it had a live cell (then
-    // it had a range), else the extension ends here
-    const bool adv = fl != 0u;
-    const int umax = int(wkey >> D::LOG2W);
-    const bool imp = adv && umax > u.X;  // S > best  <=>  S - T_d > X
-    const int d = 2 * u.e + (ODD ? 1 : 2);
-    u.bi = imp ? u.base + u.e + (ODD ? 0 : 1) + (W - 1 - int(wkey & uint32_t(W - 1))) : u.bi;
-    u.bd = imp ? d - u.phi : u.bd;
-    const int gain = imp ? umax - u.X : 0;
+    u.bd = mine ? 2 * (u.e + at) + (ODD ? 1 : 2) - u.phi : u.bd;
+    u.br = mine ? u.base + gl * C + key_slot : u.br;
     u.best += gain;
     u.theta += gain * KS + da.step;
-    // slots of the next step's frame (an even step moves rows one slot down)
-    u.lo = adv ? W - int(fl & 0xffffu) - gl * C - (ODD ? 1 : 0) : kGone;
-    u.hi = int(fl >> 16) - 1 - gl * C - (ODD ? 1 : 0);
-    if constexpr (ODD) u.mt -= 1;
-    else u.dn += 1;
+    return next_range<G, V, R, ODD>(L, ln, u.rb);
 }
 
 template <int G, int V, int R, bool UNIT>
@@ -463,17 +483,17 @@ __global__ void __launch_bounds__(128, 4)
     k_diag16(KernelArgs ka, DiagArgs da, int level, int queue, int phase) {
     const int lane = threadIdx.x & 31;
     const int gl = lane % G, unit = lane / G;
+    using D = Diag<G, V, R>;
+    const Lanes<G> ln(lane);
     const bool twin = queue != level;
     const uint32_t* q = ka.queues + size_t(queue) * ka.qcap;
     uint32_t QE[V * R], QO[V * R];
 #pragma unroll
     for (int h = 0; h < V * R; ++h) QE[h] = QO[h] = 0u;
     DState<V> u;
-    u.lo = kGone;
-    u.hi = -1;
     u.dn = u.mt = 0;
     u.theta = 32768;
-    u.best = u.bi = u.bd = u.X = 0;
+    u.best = u.bd = u.br = u.X = 0;
     u.base = u.e = u.phi = 0;
     u.c32 = 0u;
     u.cells = u.cells0 = 0ull;
@@ -481,18 +501,28 @@ __global__ void __launch_bounds__(128, 4)
     u.active = u.done = u.overflow = u.migrated = false;
 #pragma unroll
     for (int v = 0; v < V; ++v)
-        u.LE[v] = u.LO[v] = u.a0[v] = u.a1[v] = u.b0[v] = u.b1[v] = 0u;
+        u.rb[v] = u.LE[v] = u.LO[v] = u.a0[v] = u.a1[v] = u.b0[v] = u.b1[v] = 0u;
     u.na0 = u.na1 = u.nb0 = u.nb1 = 0u;
+    // the outermost slots that the next D::UNROLL steps must find dead
+    const uint32_t brink_bot = gl == 0 ? (1u << (D::UNROLL / 2)) - 1u : 0u;
+    const uint32_t brink_top = gl == G - 1 ? ((1u << (D::UNROLL / 2)) - 1u) << (D::VR - D::UNROLL / 2) : 0u;
     bool exhausted = false;
     bool first_wave = true;  // the warp's first pop takes static slots
-    int left = da.iters;
+    const int iters = da.period / D::UNROLL;  // between renormalisations
+    int left = iters;
+    uint32_t vote = 0u;  // lanes with a live slot on the last (even) anti-diagonal
     for (;;) {
-        unit_prepare<G, V, R>(ka, da, u, level, gl, unit, QE, QO);
-        if (__any_sync(FULL, u.done || (!u.active && !exhausted))) {
-            if (u.done) {
-                unit_end(ka, u, level, gl, twin);
-                u.done = false;
-            }
+        if (u.active && (vote & ln.all) == 0u) {
+            u.active = false;
+            u.done = true;
+        }
+        const bool slide = __any_sync(FULL, (u.LE[V - 1] & brink_top) != 0u || (u.LE[0] & brink_bot) != 0u);
+        if (__builtin_expect(slide, 0))
+            units_slide<G, V, R>(ka, da, u, level, gl, unit, ln, brink_top, brink_bot, QE, QO);
+        const bool turn = __any_sync(FULL, u.done || (!u.active && !exhausted));
+        if (__builtin_expect(turn, 0)) {
+            units_end<G, V>(ka, u, level, gl, twin);
+            u.done = false;
             const bool need = !u.active && !exhausted;  // the same in all lanes of a unit
             uint32_t id = 0xffffffffu;
             // one pop per warp for all of its idle units
@@ -507,13 +537,37 @@ __global__ void __launch_bounds__(128, 4)
                 if (id != 0xffffffffu) unit_start<G, V, R>(ka, da, u, id, gl, QE, QO);
                 else exhausted = true;
             }
-            if (!__any_sync(FULL, u.active)) break;
+            if (!__any_sync(FULL, u.active || u.done)) break;
         }
-        dstep<G, V, R, UNIT, true>(ka, da, u, gl, QO, QE);
-        dstep<G, V, R, UNIT, false>(ka, da, u, gl, QE, QO);
-        u.e += 1;
+        if (__builtin_expect(slide || turn, 0)) next_range<G, V, R, false>(u.LE, ln, u.rb);
+        // slots inside the matrix, rows <= m and columns <= n: step t of the
+        // loop body (t odd: an even step) has row m at mt - ceil(t / 2) and
+        // the first column at dn + floor(t / 2)
+        uint32_t inm[D::UNROLL][V];
+#pragma unroll
+        for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+            for (int v = 0; v < V; ++v) inm[t][v] = FULL;
+        if (__any_sync(FULL, u.mt < D::C + D::UNROLL / 2 || u.dn > -D::UNROLL / 2)) {
+#pragma unroll
+            for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const int k0 = __viaddmin_s32_relu(u.dn, t / 2 - v * D::VR, D::VR);
+                    const int k1 = __viaddmin_s32_relu(u.mt, 1 - (t + 1) / 2 - v * D::VR, D::VR);
+                    inm[t][v] = __funnelshift_lc(~0u, 0u, k1) & ~__funnelshift_lc(~0u, 0u, k0);
+                }
+        }
+#pragma unroll
+        for (int t = 0; t < D::UNROLL; t += 2) {
+            dstep<G, V, R, UNIT, true>(da, u, t / 2, gl, ln, inm[t], QO, QE);
+            vote = dstep<G, V, R, UNIT, false>(da, u, t / 2, gl, ln, inm[t + 1], QE, QO);
+        }
+        u.e += D::UNROLL / 2;
+        u.dn += D::UNROLL / 2;
+        u.mt -= D::UNROLL / 2;
         if (--left == 0) {
-            left = da.iters;
+            left = iters;
             unit_maintain<G, V, R>(ka, da, u, gl, QE, QO);
         }
     }
@@ -532,8 +586,8 @@ bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
         da->mp = int(mp);
         da->step = int(KS * g);
         da->floor = int(KS * grow + 64);
-        da->iters = period / 2;
-        da->unit = bonus == 2 * base ? 1 : 0;
+        da->period = period;
+        da->unit = bonus == 2 * base && mp == 1 ? 1 : 0;
         for (int p = 0; p < 6; ++p) {
             da->cb[p] = uint32_t(base) * uint32_t(KS >> p);
             da->cf[p] = uint32_t(bonus) * uint32_t(KS >> p);
@@ -545,50 +599,95 @@ bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
 
 // ---- launches ----
 
-// level -> (G, V, R) of its packed form: 32 slots per lane up to 16 lanes;
-// the 1024- and 2048-slot windows share a lane's bookkeeping between two
-// virtual lanes.
+// level -> (G, V, R) of its packed form: units of 32-slot lanes, as few as
+// the window needs (the 32-row level runs the 64-slot window too: its units
+// cost the same).  One extension per warp holds 1024 slots with one virtual
+// lane (41.6 ms on the 100,000-pair batch's level 5, against 45 with two lanes' worth of
+// rows in 16 lanes), 2048 with two.
 #define LOGAN_PACKED_LEVELS(X) \
-    X(2, 4, 1, 16) X(3, 8, 1, 16) X(4, 16, 1, 16) X(5, 16, 2, 16) X(6, 32, 2, 16)
+    X(0, 2, 1, 16) X(1, 2, 1, 16) X(2, 4, 1, 16) X(3, 8, 1, 16) X(4, 16, 1, 16) X(5, 32, 1, 16) \
+    X(6, 32, 2, 16)
 
-bool packed_level(int level) {
+bool packed_level(int level) { return level <= 6; }
+
+// the latency forms: (G, R) for windows of 128, 256 and 512 slots with 1, 2
+// or 4 extensions per warp
+#define LOGAN_PACKED_LATENCY(X) \
+    X(0, 1, 32, 2) X(0, 2, 16, 4) X(0, 4, 8, 8) X(1, 1, 32, 4) X(1, 2, 16, 8) X(2, 1, 32, 8)
+
+namespace {
+
+// resident blocks per SM, of the substitution form that needs more registers
+template <int G, int V, int R>
+int blocks_of() {
+    int a = 0, b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_diag16<G, V, R, true>, 128, 0) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_diag16<G, V, R, false>, 128, 0) !=
+            cudaSuccess)
+        return 1;
+    return std::max(1, std::min(a, b));
+}
+
+template <int G, int V, int R>
+cudaError_t launch(int level, int queue, const KernelArgs& ka, const DiagArgs& da, int grid,
+                   int phase, cudaStream_t s) {
+    if (da.unit) k_diag16<G, V, R, true><<<grid, 128, 0, s>>>(ka, da, level, queue, phase);
+    else k_diag16<G, V, R, false><<<grid, 128, 0, s>>>(ka, da, level, queue, phase);
+    return cudaGetLastError();
+}
+
+// window and units of a latency form as one number
+inline int latency_form(int level, int units) {
+    const int w = level <= 2 ? 0 : level - 2;  // levels 0-2 share the 128-slot window
+    return 10 * w + (w == 0 ? units : w == 1 ? std::min(units, 2) : 1);
+}
+
+}  // namespace
+
+int packed_level_blocks_per_sm(int level) {
     switch (level) {
-#define CASE(L, G, V, R) case L: return true;
+#define CASE(L, G, V, R) case L: return blocks_of<G, V, R>();
         LOGAN_PACKED_LEVELS(CASE)
 #undef CASE
-        default: return false;
+        default: return 0;
     }
 }
 
-cudaError_t launch_packed_level_persistent(int level, const KernelArgs& ka, const DiagArgs& da,
-                                           int grid, int phase, cudaStream_t s) {
+int packed_latency_blocks_per_sm(int level, int units) {
+    switch (latency_form(level, units)) {
+#define CASE(K, U, G, R) case 10 * K + U: return blocks_of<G, 1, R>();
+        LOGAN_PACKED_LATENCY(CASE)
+#undef CASE
+        default: return 0;
+    }
+}
+
+cudaError_t launch_packed_level(int level, const KernelArgs& ka, const DiagArgs& da, int grid,
+                                int phase, cudaStream_t s) {
     switch (level) {
-#define CASE(L, G, V, R)                                                                          \
-    case L:                                                                                       \
-        static_assert(Diag<G, V, R>::W == level_window(L), "a packed form keeps its level's window"); \
-        if (da.unit) k_diag16<G, V, R, true><<<grid, 128, 0, s>>>(ka, da, level, level, phase);   \
-        else k_diag16<G, V, R, false><<<grid, 128, 0, s>>>(ka, da, level, level, phase);          \
-        break;
+#define CASE(L, G, V, R)                                                                   \
+    case L:                                                                                \
+        static_assert(Diag<G, V, R>::W >= level_window(L) && Diag<G, V, R>::W <= mig_rows(L), \
+                      "window and record");                                                \
+        return launch<G, V, R>(level, level, ka, da, grid, phase, s);
         LOGAN_PACKED_LEVELS(CASE)
 #undef CASE
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
-int packed_level_blocks_per_sm(int level) {
-    int n = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-    switch (level) {
-#define CASE(L, G, V, R)                                                                        \
-    case L:                                                                                     \
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_diag16<G, V, R, true>, 128, 0); \
-        break;
-        LOGAN_PACKED_LEVELS(CASE)
+cudaError_t launch_packed_latency(int level, int queue, int units, const KernelArgs& ka,
+                                  const DiagArgs& da, int grid, int phase, cudaStream_t s) {
+    switch (latency_form(level, units)) {
+#define CASE(K, U, G, R)                                                                  \
+    case 10 * K + U:                                                                      \
+        static_assert(Diag<G, 1, R>::W == level_window(K + 2) && 32 / G == U, "window"); \
+        return launch<G, 1, R>(level, queue, ka, da, grid, phase, s);
+        LOGAN_PACKED_LATENCY(CASE)
 #undef CASE
-        default: break;
+        default: return cudaErrorInvalidValue;
     }
-    return e == cudaSuccess ? n : 0;
 }
 
 }  // namespace logan
