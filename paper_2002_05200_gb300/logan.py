@@ -461,15 +461,17 @@ class Context:
         n = ctypes.c_uint64()
         cr = reads.c()
         args = (self._h, ctypes.byref(cr), k, min_freq, max_freq, min_shared)
-        _check(lib().logan_overlap_candidates(*args, None, 0, ctypes.byref(n),
-                                              ctypes.c_void_p(stream.cuda_stream)),
-               "logan_overlap_candidates")
-        out = torch.empty((max(n.value, 1), 6), dtype=torch.int32, device=f"cuda:{self.device}")
-        if n.value:
-            _check(lib().logan_overlap_candidates(*args, out.data_ptr(), n.value, ctypes.byref(n),
+        # one call with room for 32 candidates a read (768 B); only a read set
+        # with more runs a second one at the size that the first returned
+        cap = max(1024, 32 * reads.count)
+        while True:
+            out = torch.empty((cap, 6), dtype=torch.int32, device=f"cuda:{self.device}")
+            _check(lib().logan_overlap_candidates(*args, out.data_ptr(), cap, ctypes.byref(n),
                                                   ctypes.c_void_p(stream.cuda_stream)),
                    "logan_overlap_candidates")
-        return out[:n.value]
+            if n.value <= cap:
+                return out[:n.value]
+            cap = n.value
 
     def overlap_pool(self, reads: DevicePool, stream=None) -> DevicePool:
         """Reads followed by their reverse complements (the extension's B side)."""
