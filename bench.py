@@ -47,10 +47,10 @@ METRIC = "X-drop GCUPS (computed cells), batched vs plain launch; serving p50/p9
 #             FMA pipe (IMAD, from sass__inst_executed_per_opcode), the rest
 #             going to the ALU pipe or to pipes that are not near a limit.
 # Reported only while the kernel's sources are the ones captured.
-PROFILED = {"level": 2, "bytes": 113.18912e6 + 9.327104e6, "items": 48_000,
-            "fma_share": 3670282022 / 11936260280,
+PROFILED = {"level": 2, "bytes": 113.513984e6 + 9.392128e6, "items": 48_000,
+            "fma_share": 3672597380 / 11914807158,
             "sources": ("xdrop_diag16.cu", "diag16.cuh", "logan_dev.cuh", "internal.h"),
-            "sha1": "f9e32405a0f43d1325eae996ddec2fc3873b986f"}
+            "sha1": "f3dcf104d615b5c4ba1320bc035564b3ed5cf500"}
 OPS_PER_CELL_AFFINE = 12  # Gotoh per cell: compare, diag add, E: 2 adds + max, F: 2 adds + max, 2 max, X-drop compare, select
 # The scope table's count for the linear recurrence, per cell: substitution
 # select, diag + substitution, max(up, left), + gap and max with the diagonal

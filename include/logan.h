@@ -327,11 +327,12 @@ int logan_overlap_keep(logan_ctx_t *ctx, const logan_result_t *results,
  *   LOGAN_ENOMEM after sizing (call again with more).
  * Work: the batch pipeline of logan_extend_batch finds every extension's
  * best cell; then each extension is swept again up to its best
- * anti-diagonal by a warp, recording 2-bit predecessor codes (a band wider
- * than 512 rows is swept by a block of 256 threads instead: in shared
- * memory up to 2048 rows, else in a device-memory ring); one thread per
- * extension walks back.  The codes take about cells / 16 words of device
- * memory -- meant for the pairs a caller keeps, not whole raw batches.
+ * anti-diagonal, recording 2-bit predecessor codes -- in the packed window
+ * that its band fitted (up to 2048 rows), else by a warp or a block of 256
+ * threads (past 2048 rows in a device-memory ring); a warp or a thread per
+ * extension walks back.  The codes take about cells / 8 words of device
+ * memory (cells / 16 when that cannot be had) -- meant for the pairs a caller
+ * keeps, not whole raw batches.
  * Temporary memory comes stream-ordered from the context's own memory pool,
  * as for logan_overlap_candidates; the call synchronises `stream` (the
  * sweeps run on `stream` and on a second stream the call creates and joins).

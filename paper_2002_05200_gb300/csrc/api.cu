@@ -209,6 +209,7 @@ void logan::extension_views(const logan_ctx_t* c, const logan_seqs_t* A, const l
     v->items = reinterpret_cast<const Item*>(w + L.items);
     v->ext = reinterpret_cast<const ExtRes*>(w + L.ext);
     v->info = reinterpret_cast<const PairInfo*>(w + L.info);
+    v->mig_slot = reinterpret_cast<const int32_t*>(w + L.mig_slot);
     v->launches = c->launches_last;
 }
 

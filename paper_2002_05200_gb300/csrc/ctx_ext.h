@@ -36,6 +36,7 @@ struct ExtensionViews {
     const Item* items = nullptr;
     const ExtRes* ext = nullptr;
     const PairInfo* info = nullptr;
+    const int32_t* mig_slot = nullptr;  // per item: the level that finished it (kMigFinal), if packed
     uint32_t launches = 0;  // kernels that call launched
 };
 void extension_views(const logan_ctx_t* c, const logan_seqs_t* A, const logan_seqs_t* B,

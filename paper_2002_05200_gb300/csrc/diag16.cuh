@@ -209,21 +209,21 @@ __device__ __forceinline__ uint32_t sign_bytes(uint32_t a, uint32_t b) {
     return r;
 }
 
-// Bit k = sign of slot k's half-word in x[0 .. R).  Four slots' sign bytes per
-// permute; for R >= 8 they are gathered by multiply-adds as 255 * mask (each
-// byte 0 or 255 times its power of two), and 255 * 0xfefefeff = 1 (mod 2^32).
+// Gathers the signs of all half-words of R registers into a mask, bit k = slot
+// k, from pairs of registers h and h + R / 2: four slots' sign bytes per
+// permute; for R >= 8 they add up by multiply-adds as 255 * mask (each byte 0
+// or 255 times its power of two), and 255 * 0xfefefeff = 1 (mod 2^32).
 template <int R>
-__device__ __forceinline__ uint32_t sign_mask(const uint32_t (&x)[R]) {
-    if constexpr (R == 2) {  // bytes: slots 0, 1, 2, 3
-        return ((sign_bytes(x[0], x[1]) & 0x08040201u) * 0x01010101u) >> 24;
-    } else if constexpr (R == 4) {  // byte j: slots 2j and 2j + 1
-        const uint32_t t = (sign_bytes(x[0], x[2]) & 0x40100401u) |
-                           (sign_bytes(x[1], x[3]) & 0x80200802u);
-        return (t * 0x01010101u) >> 24;
-    } else {
-        uint32_t acc = 0u;
-#pragma unroll
-        for (int h = 0; h < R / 2; ++h) acc = sign_bytes(x[h], x[h + R / 2]) * (1u << h) + acc;
+struct SignMask {
+    uint32_t acc = 0u;
+    __device__ __forceinline__ void add(int h, uint32_t xa, uint32_t xb) {
+        const uint32_t w = sign_bytes(xa, xb);
+        if constexpr (R == 2) acc = w & 0x08040201u;             // bytes: slots 0, 1, 2, 3
+        else if constexpr (R == 4) acc |= w & (h ? 0x80200802u : 0x40100401u);  // byte j: slots 2j, 2j + 1
+        else acc = w * (1u << h) + acc;
+    }
+    __device__ __forceinline__ uint32_t get() const {
+        if constexpr (R < 8) return (acc * 0x01010101u) >> 24;
         uint32_t m = acc * 0xfefefeffu;
         if constexpr (R == 8) {  // byte j: slots 4j .. 4j + 3, nibbles to 16 bits
             m = m | (m >> 4);
@@ -231,7 +231,7 @@ __device__ __forceinline__ uint32_t sign_mask(const uint32_t (&x)[R]) {
         }
         return m;
     }
-}
+};
 
 // bits from the highest set bit of an N-bit mask downwards (0 for 0)
 template <int N>

@@ -98,6 +98,34 @@ constexpr int kLatencyLevels = 5;
 cudaError_t launch_packed_latency(int level, int queue, int units, const KernelArgs& ka,
                                   const DiagArgs& da, int grid, int phase, cudaStream_t s);
 int packed_latency_blocks_per_sm(int level, int units);
+// Recording sweeps of the alignment paths (traceback.cu), by window class: 128,
+// 256, 512, 1024 slots in lanes of 32, 2048 in lanes of 64; a loop iteration
+// covers record_steps(c) anti-diagonals.
+constexpr int kRecordClasses = 5;
+__host__ __device__ constexpr int record_lanes(int cls) { return cls >= 3 ? 32 : 4 << cls; }
+__host__ __device__ constexpr int record_steps(int cls) { return cls == 4 ? 2 : 4; }
+// the class of an extension that ended at `level` (kRecordClasses: none)
+__host__ __device__ constexpr int record_class(int level) {
+    return level < 0 || level > 6 ? kRecordClasses : level <= 2 ? 0 : level - 2;
+}
+struct DiagRecord {
+    const uint32_t* order;     // item ids by class, the longest first
+    const uint32_t* class_at;  // class c's items are order[class_at[c] .. class_at[c + 1])
+    unsigned int* next;        // pop cursor of each class
+    const int32_t* dstar;      // per item: its best anti-diagonal
+    const uint64_t* it_off;    // per item: its first iteration in `bases`
+    const uint64_t* code_off;  // per item: its first uint4 in `codes`
+    uint4* codes;              // per iteration and lane two: (diagonal, vertical) masks of two
+                               // anti-diagonals each; lanes of 64: one per virtual lane
+    int32_t* bases;            // per iteration: the window's base
+    int32_t* outgrew;          // per item: set when its band left the window
+    unsigned int* n_outgrew;
+    unsigned long long* cells; // nullable: cells of the completed sweeps
+};
+// (bounds of its keys: packed_plan's, and no two keys 32768 apart)
+bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da);
+cudaError_t launch_record(int cls, const KernelArgs& ka, const DiagArgs& da, const DiagRecord& rc,
+                          int sms, cudaStream_t s);
 // level k's one-warp form (k < kTwinLevels), persistent over twin_queue(k)
 cudaError_t launch_twin_persistent(int level, const KernelArgs& ka, int grid, int phase,
                                    cudaStream_t s);

@@ -182,6 +182,8 @@ __device__ __forceinline__ unsigned int pop_slot(Counters* c, int q, int phase) 
 // anti-diagonal (T1 for d-1, T2 for d-2; -inf = any negative value),
 // ABSOLUTE records hold scores (-inf = NEG).
 constexpr int kMigHeader = 16;
+// mig_slot of an extension that a packed level finished: (level << 24) | kMigFinal
+constexpr unsigned int kMigFinal = 0xffffffu;
 enum MigField {
     MIG_KIND = 0, MIG_ROWS, MIG_D, MIG_BASE, MIG_LO, MIG_HI, MIG_BEST, MIG_T, MIG_T1, MIG_T2,
     MIG_BI, MIG_BJ, MIG_CELLS_LO, MIG_CELLS_HI, MIG_LEVEL

@@ -13,19 +13,25 @@
 //   1 the batch pipeline (logan_extend_batch) gives every extension its
 //     best cell (bi, bj), hence its best anti-diagonal d* = bi + bj, and its
 //     cells; its workspace keeps the packed sequences and the split items;
-//   2 per extension the storage of its predecessor codes: every
-//     anti-diagonal 1..d* starts on a 16-cell word, so cells / 16 + d* + 1
-//     words suffice; scans give the offsets;
-//   3 the sweep again up to d*, one warp per extension with its three
-//     anti-diagonals in a shared-memory ring of 512 rows (a band that
-//     outgrows it runs again on a block of 256 threads: 2048 rows in shared
-//     memory, else a device-memory ring -- the paper's layout, Sec. IV-B),
-//     writing for every anti-diagonal its first row, its first word and the
-//     2-bit codes of its cells (16 lanes' codes ORed into a word by warp
-//     reductions);
-//   4 one thread per extension walks back from its best cell (run-length
-//     codes, length << 4 | op; op 0 = M, 1 = I, 2 = D), one thread per pair
-//     joins the left codes, the seed and the right codes.
+//   2 extensions that a packed level finished are swept again by its recording
+//     form (xdrop_diag16.cu) in a window as wide as the level's, up to d*:
+//     fixed storage of two bits per window slot and anti-diagonal; the bands
+//     that leave the window (it fitted at other offsets) go to the next wider
+//     one in a second round.  10,000 lognormal pairs: 49 ms of recording, against
+//     141 ms with step 3 for all;
+//   3 the rest (scores or X past 16 bits, bands past 2048 rows, no memory for
+//     step 2's codes): per extension the storage of its codes, every
+//     anti-diagonal 1..d* starting on a 16-cell word, so cells / 16 + d* + 1
+//     words suffice; one warp per extension with its three anti-diagonals in
+//     a shared-memory ring of 512 rows (a band that outgrows it runs again on
+//     a block of 256 threads: 2048 rows in shared memory, else a
+//     device-memory ring -- the paper's layout, Sec. IV-B), writing for every
+//     anti-diagonal its first row, its first word and the 2-bit codes of its
+//     cells (16 lanes' codes ORed into a word by warp reductions);
+//   4 a warp (step 2's codes) or a thread (step 3's) per extension walks back
+//     from its best cell (run-length codes, length << 4 | op; op 0 = M, 1 = I,
+//     2 = D), one thread per pair joins the left codes, the seed and the right
+//     codes.
 // Same cell update and range rules as the extension kernels, so the sweep
 // meets the same best cells.
 #include <cub/device/device_radix_sort.cuh>
@@ -57,6 +63,7 @@ constexpr int TB_WIDE = 1;       // status: retry in the device-memory ring
 constexpr int TB_WARP_WIDE = 2;  // status: wide from the start, swept by a block
 constexpr int TB_BOUND = 3;      // status: the codes outgrew the item's words (not expected)
 constexpr int TB_OUTGREW = 4;    // status: outgrew a warp's ring, retry on a block
+constexpr int TB_DIAG = 2;       // `wide` - TB_DIAG: class of the packed sweep that recorded it (xdrop_diag16.cu)
 
 struct TbRed {
     int mx, first, last;
@@ -79,7 +86,7 @@ __device__ __forceinline__ TbRed tb_reduce(TbRed v, TbRed* sh) {
 
 struct TbItem {  // per item: its best cell and the recording sweep's status
     int32_t bi, bj, status;
-    int32_t wide;  // swept by a block from the start (the warp sweep leaves it alone)
+    int32_t wide;  // 1: swept by a block from the start, >= TB_DIAG: a packed sweep (the warp sweep leaves both alone)
 };
 
 struct TbArgs {
@@ -94,6 +101,7 @@ struct TbArgs {
     unsigned long long* cells; // nullable: cells of the completed sweeps
     const uint32_t* order;     // item ids, the most code words first
     unsigned int* next;        // pop cursors into order: [0] warps, [1] and [2] the block passes
+    DiagRecord rec;            // the packed sweeps' codes
 };
 
 // The sweep of one item up to its best anti-diagonal by TW threads (a warp,
@@ -268,13 +276,17 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_record_block(TbArgs t, int wh
     }
 }
 
-// Per item from the extension's results: best cell, status and sizes (code
-// words, anti-diagonal table entries); per pair the run-length codes bound.
+// Per item from the extension's results: best cell, status, the window class
+// whose recording sweep takes it (kRecordClasses: the general sweep), and
+// that sweep's sizes (loop iterations, 16-byte code groups); per class its
+// items; per pair the run-length codes bound.
 __global__ void k_tb_prepare(const Item* __restrict__ items, const ExtRes* __restrict__ ext,
-                             const PairInfo* __restrict__ pi,
-                             const uint32_t* __restrict__ seeds, uint32_t n_pairs,
-                             TbItem* __restrict__ info, uint64_t* __restrict__ item_words,
-                             uint64_t* __restrict__ item_ads, uint64_t* __restrict__ pair_codes) {
+                             const PairInfo* __restrict__ pi, const int32_t* __restrict__ mig_slot,
+                             const uint32_t* __restrict__ seeds, uint32_t n_pairs, int32_t record_x,
+                             TbItem* __restrict__ info, int32_t* __restrict__ dstar_out,
+                             uint64_t* __restrict__ order_key, uint64_t* __restrict__ iters,
+                             uint64_t* __restrict__ groups, uint64_t* __restrict__ pair_codes,
+                             uint64_t* __restrict__ side_n, unsigned int* __restrict__ class_n) {
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n_pairs;
          p += gridDim.x * blockDim.x) {
         uint64_t codes = 1;
@@ -282,26 +294,92 @@ __global__ void k_tb_prepare(const Item* __restrict__ items, const ExtRes* __res
             const uint32_t id = 2 * p + s;
             const ExtRes e = ext[id];
             const int32_t st = pi[p].status ? pi[p].status : e.status;
-            TbItem x{st ? 0 : e.bi, st ? 0 : e.bj, st, 0};
-            const uint64_t dstar = uint64_t(x.bi) + uint64_t(x.bj);
-            // a sweep of at most m + n anti-diagonals whose cells average
-            // more than kWarpCap / 2 per anti-diagonal is swept by a block
-            // from the start (a warp would outgrow its ring)
-            const Item it = items[id];
-            if (!st && dstar &&
-                uint64_t(e.cells) > uint64_t(kWarpCap / 2) * (uint64_t(it.m) + uint64_t(it.n))) {
-                x.status = TB_WARP_WIDE;
-                x.wide = 1;
+            const int32_t bi = st ? 0 : e.bi, bj = st ? 0 : e.bj;
+            const int32_t dstar = bi + bj;
+            int cls = kRecordClasses;
+            if (!st && dstar && items[id].X <= record_x) {
+                const int32_t m = mig_slot[id];
+                if (m >= 0 && (uint32_t(m) & kMigFinal) == kMigFinal) cls = record_class(m >> 24);
             }
-            info[id] = x;
-            // anti-diagonals 1..d* hold at most the extension's cells, each
-            // starting on a word
-            item_words[id] = dstar ? uint64_t(e.cells) / 16u + dstar + 1u : 0u;
-            item_ads[id] = dstar + 1u;
-            codes += dstar;
+            info[id] = TbItem{bi, bj, st, cls < kRecordClasses ? TB_DIAG + cls : 0};
+            dstar_out[id] = dstar;
+            order_key[id] = (uint64_t(cls) << 32) | (0xffffffffu - uint32_t(dstar));
+            const uint64_t steps = uint64_t(record_steps(cls));
+            const uint64_t n = cls < kRecordClasses ? (uint64_t(dstar) + steps - 1u) / steps : 0u;
+            iters[id] = n;
+            groups[id] = n * 2u * uint64_t(record_lanes(cls));
+            if (cls < kRecordClasses || dstar) atomicAdd(&class_n[cls], 1u);
+            codes += uint64_t(dstar);
         }
-        pair_codes[p] = codes + seeds[5 * p + 4];
+        codes += seeds[5 * p + 4];
+        pair_codes[p] = codes;
+        // (a side without a path has nothing to walk: no codes at its end of the region)
+        if (info[2 * p].bi + info[2 * p].bj == 0) side_n[2 * p] = 0u;
+        if (info[2 * p + 1].bi + info[2 * p + 1].bj == 0) side_n[2 * p + 1] = codes;
     }
+}
+
+// Second round: the items whose band left their window move to the next wider
+// class (the widest ones' to the general sweep), the others have none.
+__global__ void k_tb_wider(const int32_t* __restrict__ outgrew, const int32_t* __restrict__ dstar,
+                           uint32_t n_items, TbItem* __restrict__ info,
+                           uint64_t* __restrict__ order_key, uint64_t* __restrict__ iters,
+                           uint64_t* __restrict__ groups, unsigned int* __restrict__ class_n) {
+    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= n_items) return;
+    int cls = kRecordClasses;
+    if (outgrew[id]) {
+        cls = info[id].wide - TB_DIAG + 1;
+        info[id].wide = cls < kRecordClasses ? TB_DIAG + cls : 0;
+        atomicAdd(&class_n[cls], 1u);
+    }
+    order_key[id] = (uint64_t(cls) << 32) | (0xffffffffu - uint32_t(dstar[id]));
+    const uint64_t steps = uint64_t(record_steps(cls));
+    const uint64_t n = cls < kRecordClasses ? (uint64_t(dstar[id]) + steps - 1u) / steps : 0u;
+    iters[id] = n;
+    groups[id] = n * 2u * uint64_t(record_lanes(cls));
+}
+
+// first item of each class in the sorted order
+__global__ void k_tb_class_at(const unsigned int* __restrict__ class_n, uint32_t* __restrict__ class_at) {
+    uint32_t at = 0;
+    for (int c = 0; c <= kRecordClasses; ++c) {
+        class_at[c] = at;
+        if (c < kRecordClasses) at += class_n[c];
+    }
+}
+
+// The items left for the general sweep: those without a class (all when
+// `every`) and those whose band left its window; their sizes (code words,
+// anti-diagonal table entries), 0 for the others.
+__global__ void k_tb_general(const Item* __restrict__ items, const ExtRes* __restrict__ ext,
+                             uint32_t n_items, const int32_t* __restrict__ outgrew, int every,
+                             TbItem* __restrict__ info, uint64_t* __restrict__ item_words,
+                             uint64_t* __restrict__ item_ads) {
+    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= n_items) return;
+    TbItem x = info[id];
+    const uint64_t dstar = uint64_t(x.bi) + uint64_t(x.bj);
+    if (x.wide >= TB_DIAG && !every && !outgrew[id]) {
+        item_words[id] = 0u;
+        item_ads[id] = 0u;
+        return;
+    }
+    x.wide = 0;
+    // a sweep of at most m + n anti-diagonals whose cells average more than
+    // kWarpCap / 2 per anti-diagonal is swept by a block from the start (a warp
+    // would outgrow its ring)
+    const Item it = items[id];
+    const uint64_t cells = ext[id].cells;
+    if (!x.status && dstar && cells > uint64_t(kWarpCap / 2) * (uint64_t(it.m) + uint64_t(it.n))) {
+        x.status = TB_WARP_WIDE;
+        x.wide = 1;
+    }
+    info[id] = x;
+    // anti-diagonals 1..d* hold at most the extension's cells, each starting
+    // on a word
+    item_words[id] = dstar ? cells / 16u + dstar + 1u : 0u;
+    item_ads[id] = dstar + 1u;
 }
 
 __global__ void k_tb_iota(uint32_t* __restrict__ ids, uint32_t n) {
@@ -335,16 +413,28 @@ __global__ void k_tb_walk(TbArgs t, const uint32_t* __restrict__ seeds, uint32_t
         const bool right = (id & 1u) != 0u;
         const TbItem x = t.info[id];
         const TbItem o = t.info[id ^ 1u];
-        if (x.status || o.status) continue;
+        if (x.status || o.status || x.wide >= TB_DIAG) continue;
         uint32_t* region = ops + op_start[p];
         const TbItem& L = right ? o : x;
         const TbItem& Rr = right ? x : o;
         const uint64_t bound = uint64_t(L.bi) + L.bj + seeds[5 * p + 4] + Rr.bi + Rr.bj + 1;
         uint64_t at = right ? bound : 0;
         int i = x.bi, d = x.bi + x.bj;
-        const uint64_t ab = t.ad_off[id];
         uint32_t cur = 3u, len = 0;
+        auto step = [&](uint32_t h) {
+            if (h == cur) {
+                ++len;
+                return;
+            }
+            if (len) {
+                if (right) region[--at] = (len << 4) | cur;
+                else region[at++] = (len << 4) | cur;
+            }
+            cur = h;
+            len = 1;
+        };
         if (d > 0) {
+            const uint64_t ab = t.ad_off[id];
             int rlo = t.ad_rlo[ab + d];
             uint64_t word = t.ad_word[ab + d];
             while (d > 0) {
@@ -354,16 +444,7 @@ __global__ void k_tb_walk(TbArgs t, const uint32_t* __restrict__ seeds, uint32_t
                 const int r1 = t.ad_rlo[ab + d1], r2 = t.ad_rlo[ab + d2];
                 const uint64_t w1 = t.ad_word[ab + d1], w2 = t.ad_word[ab + d2];
                 const uint32_t h = tb_code(t, rlo, word, i);
-                if (h == cur) {
-                    ++len;
-                } else {
-                    if (len) {
-                        if (right) region[--at] = (len << 4) | cur;
-                        else region[at++] = (len << 4) | cur;
-                    }
-                    cur = h;
-                    len = 1;
-                }
+                step(h);
                 if (h == 0u) {
                     --i;
                     d = d2;
@@ -383,6 +464,90 @@ __global__ void k_tb_walk(TbArgs t, const uint32_t* __restrict__ seeds, uint32_t
         }
         side_n[id] = at;
     }
+}
+
+// The same walk for the extensions that a packed sweep recorded, a warp each.
+// The path stays in a lane's slots for long (the frame follows the main
+// diagonal), so the warp loads that lane's codes of 16 loop iterations at once
+// (half an iteration per thread) and the moves read them by shuffles: about 90
+// cycles each, where a thread per walk waited for a load at every move
+// whenever any of its warp's 32 walks did.
+__global__ void __launch_bounds__(128) k_tb_walk_diag(TbArgs t, const uint32_t* __restrict__ seeds,
+                                                      uint32_t n_items,
+                                                      const uint64_t* __restrict__ op_start,
+                                                      uint32_t* __restrict__ ops,
+                                                      uint64_t* __restrict__ side_n) {
+    const int me = int(threadIdx.x & 31u);
+    const uint32_t slot_id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (slot_id >= t.rec.class_at[kRecordClasses]) return;
+    const uint32_t id = t.rec.order[slot_id];
+    const TbItem x = t.info[id], o = t.info[id ^ 1u];
+    // (left to the second round or the general sweep)
+    if (x.status || o.status || x.wide < TB_DIAG || t.rec.outgrew[id]) return;
+    const int cls = x.wide - TB_DIAG;
+    const int lanes = record_lanes(cls), log_steps = record_steps(cls) == 4 ? 2 : 1;
+    const int log_rows = log_steps == 2 ? 5 : 6;  // slots of a lane
+    const uint32_t p = id >> 1;
+    const bool right = (id & 1u) != 0u;
+    uint32_t* region = ops + op_start[p];
+    const TbItem& L = right ? o : x;
+    const TbItem& Rr = right ? x : o;
+    const uint64_t bound = uint64_t(L.bi) + L.bj + seeds[5 * p + 4] + Rr.bi + Rr.bj + 1;
+    uint64_t at = right ? bound : 0;
+    const uint4* codes = t.rec.codes + t.rec.code_off[id];
+    const int32_t* bases = t.rec.bases + t.rec.it_off[id];
+    int i = x.bi, d = x.bi + x.bj;
+    uint32_t cur = 3u, len = 0;
+    int top = -1, lane = -1;  // the loaded lane's iterations top, top - 1, .., top - 15
+    int32_t base = 0;         // this thread's iteration: top - me / 2
+    uint4 c{};
+    while (d > 0) {
+        const int it = (d - 1) >> log_steps, st = (d - 1) & ((1 << log_steps) - 1);
+        if (it > top || it <= top - 16) {  // (d only falls, so a batch is left downwards)
+            top = it;
+            lane = -1;
+            base = top - (me >> 1) >= 0 ? bases[top - (me >> 1)] : 0;
+        }
+        const int src = 2 * (top - it);
+        const int slot = i - (d >> 1) - __shfl_sync(FULL, base, src);
+        if ((slot >> log_rows) != lane) {
+            lane = slot >> log_rows;
+            const int mine = top - (me >> 1);
+            if (mine >= 0) c = codes[(size_t(mine) * lanes + lane) * 2 + (me & 1)];
+        }
+        // two anti-diagonals of a lane per 16 bytes, or a virtual lane's
+        const int half = log_steps == 2 ? st >> 1 : (slot >> 5) & 1;
+        const uint32_t dg = __shfl_sync(FULL, (st & 1) ? c.z : c.x, src + half);
+        const uint32_t up = __shfl_sync(FULL, (st & 1) ? c.w : c.y, src + half);
+        const uint32_t b = uint32_t(slot) & 31u;
+        const uint32_t h = ((dg >> b) & 1u) ? 0u : ((up >> b) & 1u) ? 1u : 2u;
+        if (h == cur) {
+            ++len;
+        } else {
+            if (len) {
+                if (right) --at;
+                if (me == 0) region[at] = (len << 4) | cur;
+                if (!right) ++at;
+            }
+            cur = h;
+            len = 1;
+        }
+        i -= h != 2u ? 1 : 0;
+        d -= h == 0u ? 2 : 1;
+    }
+    if (len) {
+        if (right) --at;
+        if (me == 0) region[at] = (len << 4) | cur;
+        if (!right) ++at;
+    }
+    if (me == 0) side_n[id] = at;
+}
+
+__global__ void k_tb_clear(unsigned int* __restrict__ counts, int n_counts,
+                           int32_t* __restrict__ outgrew, uint32_t n_items) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < uint32_t(n_counts)) counts[i] = 0u;
+    if (i < n_items) outgrew[i] = 0;
 }
 
 struct RleOut {
@@ -442,6 +607,16 @@ struct TbScratch {
         ptrs.push_back(p);
         return static_cast<T*>(p);
     }
+    // null instead of failing the call
+    template <typename T>
+    T* try_get(size_t n) {
+        T* p = get<T>(n);
+        if (!p) {
+            ok = true;
+            (void)cudaGetLastError();
+        }
+        return p;
+    }
     ~TbScratch() {
         // (after an error between the fork and the join, aux may still run)
         if (aux) cudaStreamSynchronize(aux);
@@ -452,7 +627,8 @@ struct TbScratch {
     }
 };
 
-// exclusive prefix of v[0, n) into out[0, n]; returns out[n] (synchronises)
+// exclusive prefix of v[0, n) into out[0, n]; *total gets out[n] once the
+// stream has synchronised
 bool tb_scan(TbScratch& sc, uint64_t* v, uint64_t n, uint64_t* out, uint64_t* total) {
     cudaMemsetAsync(v + n, 0, sizeof(uint64_t), sc.s);
     size_t tb = 0;
@@ -461,8 +637,25 @@ bool tb_scan(TbScratch& sc, uint64_t* v, uint64_t n, uint64_t* out, uint64_t* to
     if (!sc.ok) return false;
     cub::DeviceScan::ExclusiveSum(tmp, tb, v, out, n + 1, sc.s);
     return cudaMemcpyAsync(total, out + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, sc.s) ==
-               cudaSuccess &&
-           cudaStreamSynchronize(sc.s) == cudaSuccess;
+           cudaSuccess;
+}
+
+// ids[0, n) ordered by descending keys (ascending = false) or ascending ones
+bool tb_order(TbScratch& sc, const uint64_t* keys, uint32_t n, bool ascending, uint32_t* order) {
+    uint32_t* ids = sc.get<uint32_t>(n);
+    uint64_t* sorted = sc.get<uint64_t>(n);
+    size_t bytes = 0;
+    auto sort = [&](void* tmp) {
+        return ascending ? cub::DeviceRadixSort::SortPairs(tmp, bytes, keys, sorted, ids, order, int(n), 0,
+                                                           36, sc.s)
+                         : cub::DeviceRadixSort::SortPairsDescending(tmp, bytes, keys, sorted, ids, order,
+                                                                     int(n), 0, 64, sc.s);
+    };
+    sort(nullptr);
+    void* tmp = sc.get<char>(bytes);
+    if (!sc.ok) return false;
+    k_tb_iota<<<(n + 255) / 256, 256, 0, sc.s>>>(ids, n);
+    return sort(tmp) == cudaSuccess;
 }
 
 // CUDA events around the steps of one timed call (LOGAN_OPT_TIMING)
@@ -504,29 +697,25 @@ struct TbClock {
     }
 };
 
-int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seeds,
-                  uint32_t n_pairs, Scoring sc, uint32_t ring_log2, uint32_t* ops,
-                  uint64_t capacity, uint64_t* op_start, uint32_t* op_count, uint64_t* needed,
-                  cudaStream_t s, TbScratch& S, TbClock& clk) {
-    const uint32_t n_items = 2u * n_pairs;
-    const uint32_t* sd = reinterpret_cast<const uint32_t*>(seeds);
-    TbItem* tinfo = S.get<TbItem>(n_items);
+// The general sweeps of the items that the packed ones leave (all when
+// `every`): sizes, storage, one warp per item, a block for the wide bands.
+int run_general(int num_sms, const ExtensionViews& v, uint32_t n_items, Scoring sc,
+                uint32_t ring_log2, bool every, TbItem* tinfo, const int32_t* outgrew, TbArgs& t,
+                cudaStream_t s, TbScratch& S, TbClock& clk) {
     uint64_t* iw = S.get<uint64_t>(n_items + 1);
     uint64_t* ia = S.get<uint64_t>(n_items + 1);
-    uint64_t* pc = S.get<uint64_t>(n_pairs + 1);
     uint64_t* woff = S.get<uint64_t>(n_items + 1);
     uint64_t* aoff = S.get<uint64_t>(n_items + 1);
-    uint64_t* side_n = S.get<uint64_t>(n_items);
+    uint32_t* order = S.get<uint32_t>(n_items);
+    unsigned int* next = S.get<unsigned int>(3);
     if (!S.ok) return LOGAN_ENOMEM;
-    k_tb_prepare<<<(n_pairs + 255) / 256, 256, 0, s>>>(v.items, v.ext, v.info, sd, n_pairs,
-                                                       tinfo, iw, ia, pc);
+    k_tb_general<<<(n_items + 255) / 256, 256, 0, s>>>(v.items, v.ext, n_items, outgrew, every ? 1 : 0,
+                                                       tinfo, iw, ia);
     ++clk.launches;
-    uint64_t total_words = 0, total_ads = 0, total_codes = 0;
+    uint64_t total_words = 0, total_ads = 0;
     if (!tb_scan(S, iw, n_items, woff, &total_words) || !tb_scan(S, ia, n_items, aoff, &total_ads) ||
-        !tb_scan(S, pc, n_pairs, op_start, &total_codes))
+        cudaStreamSynchronize(s) != cudaSuccess)
         return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
-    *needed = total_codes;
-    if (capacity < total_codes) return LOGAN_ENOMEM;
     // 8 blocks of 256 threads fill an SM (24 KB of shared ring each)
     const int grid = int(std::min<uint32_t>(n_items, uint32_t(num_sms) * 8u));
     const int wgrid = int(std::min<uint32_t>((n_items + kTbWarps - 1) / kTbWarps,
@@ -536,46 +725,23 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
     uint32_t* codes = S.get<uint32_t>(total_words);
     int32_t* ad_rlo = S.get<int32_t>(total_ads);
     uint64_t* ad_word = S.get<uint64_t>(total_ads);
-    if (clk.on) clk.dcells = S.get<unsigned long long>(1);
     if (!S.ok) return LOGAN_ENOMEM;
     // the recording sweeps pop the items the most code words first
-    uint32_t* ids = S.get<uint32_t>(n_items);
-    uint32_t* order = S.get<uint32_t>(n_items);
-    uint64_t* keys = S.get<uint64_t>(n_items);
-    unsigned int* next = S.get<unsigned int>(3);
-    size_t sort_bytes = 0;
-    cub::DeviceRadixSort::SortPairsDescending(nullptr, sort_bytes, iw, keys, ids, order,
-                                              int(n_items), 0, 64, s);
-    void* sort_tmp = S.get<char>(sort_bytes);
-    if (!S.ok) return LOGAN_ENOMEM;
-    k_tb_iota<<<(n_items + 255) / 256, 256, 0, s>>>(ids, n_items);
+    if (!tb_order(S, iw, n_items, false, order)) return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
     ++clk.launches;
-    if (cub::DeviceRadixSort::SortPairsDescending(sort_tmp, sort_bytes, iw, keys, ids, order,
-                                                  int(n_items), 0, 64, s) != cudaSuccess)
-        return LOGAN_ECUDA;
     cudaMemsetAsync(next, 0, 3 * sizeof(unsigned int), s);
     cudaMemsetAsync(ad_rlo, 0, sizeof(int32_t) * std::max<uint64_t>(total_ads, 1), s);
     cudaMemsetAsync(ad_word, 0, sizeof(uint64_t) * std::max<uint64_t>(total_ads, 1), s);
-    if (clk.dcells) cudaMemsetAsync(clk.dcells, 0, sizeof(unsigned long long), s);
-    TbArgs t{};
-    t.ka.wa = v.wa;
-    t.ka.wb = v.wb;
-    t.ka.items = v.items;
     t.ka.ring = ring;
     t.ka.ring_cap = cap;
-    t.ka.n_items = n_items;
-    t.ka.sc = sc;
-    t.info = tinfo;
     t.word_off = woff;
     t.ad_off = aoff;
     t.codes = codes;
     t.ad_rlo = ad_rlo;
     t.ad_word = ad_word;
     t.n_words = total_words;
-    t.cells = clk.dcells;
     t.order = order;
     t.next = next;
-    clk.mark(TbClock::REC_START, s);
     // the block sweep of the items wide from the start runs beside the warp
     // sweep (it holds a few SMs for long, the warp sweep fills the rest); the
     // block sweep of the items that outgrew a warp's ring follows both
@@ -586,13 +752,156 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
     if (cudaEventRecord(S.join, S.aux) != cudaSuccess || cudaStreamWaitEvent(s, S.join, 0) != cudaSuccess)
         return LOGAN_ECUDA;
     k_tb_record_block<<<grid, kTbThreads, 0, s>>>(t, TB_OUTGREW, 2);
+    clk.launches += 3;
+    clk.words += total_words;
+    return LOGAN_OK;
+}
+
+int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seeds,
+                  uint32_t n_pairs, Scoring sc, int32_t X, bool per_pair_x, uint32_t ring_log2,
+                  uint32_t* ops, uint64_t capacity, uint64_t* op_start, uint32_t* op_count,
+                  uint64_t* needed, cudaStream_t s, TbScratch& S, TbClock& clk) {
+    const uint32_t n_items = 2u * n_pairs;
+    const uint32_t* sd = reinterpret_cast<const uint32_t*>(seeds);
+    // the largest X whose keys the packed recording sweeps hold: the call's, or
+    // with X per pair the upper bound of an X class (others take the general sweep)
+    DiagArgs da{};
+    int32_t record_x = -1;
+    for (int32_t x : {per_pair_x ? 700 : X, 300, 150, 75}) {
+        if (!per_pair_x && x != X) break;
+        if (record_plan(sc, x, &da)) {
+            record_x = x;
+            break;
+        }
+    }
+    TbItem* tinfo = S.get<TbItem>(n_items);
+    int32_t* dstar = S.get<int32_t>(n_items);
+    uint64_t* pc = S.get<uint64_t>(n_pairs + 1);
+    uint64_t* side_n = S.get<uint64_t>(n_items);
+    if (clk.on) clk.dcells = S.get<unsigned long long>(1);
+    if (!S.ok) return LOGAN_ENOMEM;
+    if (clk.dcells) cudaMemsetAsync(clk.dcells, 0, sizeof(unsigned long long), s);
+    TbArgs t{};
+    t.ka.wa = v.wa;
+    t.ka.wb = v.wb;
+    t.ka.items = v.items;
+    t.ka.n_items = n_items;
+    t.ka.sc = sc;
+    t.ka.one = 1;
+    t.info = tinfo;
+    t.cells = clk.dcells;
+    // The packed sweeps: fixed storage per window slot, about twice what the
+    // general sweep's takes (without room for it, the general sweep takes all).
+    // A second round takes the bands that left their window to the next
+    // wider one.
+    struct Round {
+        uint64_t *key, *iters, *groups, *it_off, *code_off;
+        unsigned int* counts;  // items per class, pop cursors, the number that left their window
+        uint32_t *class_at, *order;
+        int32_t* outgrew;
+        DiagRecord rec;
+        uint32_t items = 0;
+    } rounds[2];
+    constexpr int kCounts = 2 * kRecordClasses + 2;
+    bool every = false;
+    uint32_t rest = 0;
+    int n_rounds = 0;
+    for (int r = 0; r < 2; ++r) {
+        Round& q = rounds[r];
+        q.key = S.get<uint64_t>(n_items);
+        q.iters = S.get<uint64_t>(n_items + 1);
+        q.groups = S.get<uint64_t>(n_items + 1);
+        q.it_off = S.get<uint64_t>(n_items + 1);
+        q.code_off = S.get<uint64_t>(n_items + 1);
+        q.counts = S.get<unsigned int>(kCounts);
+        q.class_at = S.get<uint32_t>(kRecordClasses + 1);
+        q.order = S.get<uint32_t>(n_items);
+        q.outgrew = S.get<int32_t>(n_items);
+        q.rec = DiagRecord{};
+        if (!S.ok) return LOGAN_ENOMEM;
+        k_tb_clear<<<(std::max<uint32_t>(n_items, kCounts) + 255) / 256, 256, 0, s>>>(
+            q.counts, kCounts, q.outgrew, n_items);
+        if (r == 0)
+            k_tb_prepare<<<(n_pairs + 255) / 256, 256, 0, s>>>(
+                v.items, v.ext, v.info, v.mig_slot, sd, n_pairs, record_x, tinfo, dstar, q.key, q.iters,
+                q.groups, pc, side_n, q.counts);
+        else
+            k_tb_wider<<<(n_items + 255) / 256, 256, 0, s>>>(rounds[0].outgrew, dstar, n_items, tinfo,
+                                                             q.key, q.iters, q.groups, q.counts);
+        k_tb_class_at<<<1, 1, 0, s>>>(q.counts, q.class_at);
+        clk.launches += 3;
+        uint64_t total_it = 0, total_groups = 0, total_codes = 0;
+        unsigned int n_class[kRecordClasses + 1] = {};
+        if (!tb_scan(S, q.iters, n_items, q.it_off, &total_it) ||
+            !tb_scan(S, q.groups, n_items, q.code_off, &total_groups) ||
+            (r == 0 && !tb_scan(S, pc, n_pairs, op_start, &total_codes)))
+            return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
+        if (cudaMemcpyAsync(n_class, q.counts, sizeof(n_class), cudaMemcpyDeviceToHost, s) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return LOGAN_ECUDA;
+        if (r == 0) {
+            *needed = total_codes;
+            if (capacity < total_codes) return LOGAN_ENOMEM;
+            clk.mark(TbClock::REC_START, s);
+        }
+        rest += n_class[kRecordClasses];
+        for (int c = 0; c < kRecordClasses; ++c) q.items += n_class[c];
+        if (!q.items) break;
+        uint4* codes = S.try_get<uint4>(total_groups);
+        int32_t* bases = codes ? S.try_get<int32_t>(total_it) : nullptr;
+        if (!bases) {
+            every = true;
+            break;
+        }
+        if (!tb_order(S, q.key, n_items, true, q.order)) return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
+        q.rec = DiagRecord{q.order, q.class_at, q.counts + kRecordClasses + 1, dstar, q.it_off,
+                           q.code_off, codes, bases, q.outgrew, q.counts + 2 * kRecordClasses + 1,
+                           clk.dcells};
+        // the wide classes, fewer and slower, beside the narrow one
+        if (cudaEventRecord(S.fork, s) != cudaSuccess ||
+            cudaStreamWaitEvent(S.aux, S.fork, 0) != cudaSuccess)
+            return LOGAN_ECUDA;
+        for (int c = kRecordClasses - 1; c >= 0; --c) {
+            if (!n_class[c]) continue;
+            if (launch_record(c, t.ka, da, q.rec, num_sms, c ? S.aux : s) != cudaSuccess)
+                return LOGAN_ECUDA;
+            ++clk.launches;
+        }
+        unsigned int n_out = 0;
+        if (cudaEventRecord(S.join, S.aux) != cudaSuccess ||
+            cudaStreamWaitEvent(s, S.join, 0) != cudaSuccess ||
+            cudaMemcpyAsync(&n_out, q.rec.n_outgrew, sizeof(n_out), cudaMemcpyDeviceToHost, s) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return LOGAN_ECUDA;
+        clk.launches += 1;
+        clk.words += total_groups * 4u + total_it;
+        n_rounds = r + 1;
+        if (!n_out) break;
+        if (r == 1) rest += n_out;
+    }
+    const int32_t* outgrew = rounds[n_rounds ? n_rounds - 1 : 0].outgrew;
+    if (rest || every) {
+        const int rc = run_general(num_sms, v, n_items, sc, ring_log2, every, tinfo, outgrew, t, s, S, clk);
+        if (rc != LOGAN_OK) return rc;
+    }
     clk.mark(TbClock::REC_END, s);
-    k_tb_walk<<<(n_items + 127) / 128, 128, 0, s>>>(t, sd, n_pairs, op_start, ops, side_n);
+    // one warp per packed-recorded extension (longest first within a class),
+    // one thread per other one
+    for (int r = 0; r < n_rounds && !every; ++r) {
+        t.rec = rounds[r].rec;
+        k_tb_walk_diag<<<(rounds[r].items + 3) / 4, 128, 0, s>>>(t, sd, n_items, op_start, ops, side_n);
+        ++clk.launches;
+    }
+    if (rest || every || !n_rounds) {
+        k_tb_walk<<<(n_items + 127) / 128, 128, 0, s>>>(t, sd, n_pairs, op_start, ops, side_n);
+        ++clk.launches;
+    }
     k_tb_join<<<(n_pairs + 127) / 128, 128, 0, s>>>(tinfo, sd, n_pairs, op_start, ops, side_n,
                                                     op_count);
     clk.mark(TbClock::END, s);
-    clk.launches += 5;
-    clk.words = total_words;
+    clk.launches += 1;
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess)
         return LOGAN_ECUDA;
     return LOGAN_OK;
@@ -649,8 +958,8 @@ extern "C" int logan_traceback_batch(logan_ctx_t* ctx, const logan_seqs_t* A,
             ExtensionViews v;
             extension_views(ctx, A, B, n_pairs, ws, &v);
             clk.launches += v.launches;
-            rc = run_traceback(sms, v, seeds, n_pairs, Scoring{match, mismatch, gap},
-                               uint32_t(ring_log2), ops, ops_capacity, op_start, op_count,
+            rc = run_traceback(sms, v, seeds, n_pairs, Scoring{match, mismatch, gap}, X,
+                               X_per_pair != nullptr, uint32_t(ring_log2), ops, ops_capacity, op_start, op_count,
                                ops_needed, s, S, clk);
         }
         if (rc == LOGAN_OK && clk.on) {

@@ -39,7 +39,8 @@ namespace logan {
 
 namespace {
 
-template <int G, int V, int R>
+// (FRESH: from the extension's start, whatever records exist)
+template <int G, int V, int R, bool FRESH = false>
 __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
                                            uint32_t id, int gl, uint32_t (&QE)[V * R],
                                            uint32_t (&QO)[V * R]) {
@@ -50,8 +51,11 @@ __device__ __forceinline__ void unit_start(const KernelArgs& ka, const DiagArgs&
     u.c32 = 0u;
     u.theta = 32768;
     bool fits = true;
-    const int32_t slot = ka.mig_slot[id];
-    const int32_t* rec = slot >= 0 ? mig_record(ka, slot) : nullptr;
+    const int32_t* rec = nullptr;
+    if constexpr (!FRESH) {
+        const int32_t slot = ka.mig_slot[id];
+        if (slot >= 0) rec = mig_record(ka, slot);
+    }
     if (rec && rec[MIG_KIND] == MIG_RELATIVE) {
         // resume a band saved by a narrower level
         const int rows = rec[MIG_ROWS], d = rec[MIG_D], row0 = rec[MIG_BASE];
@@ -164,6 +168,10 @@ __device__ __forceinline__ void units_end(const KernelArgs& ka, DState<V>& u, in
         r.status = 0;
         r.cells = u.cells0 + cells;
         ka.ext[u.item] = r;
+        // (the item's record, if it had one, has been read) the level whose
+        // window held the band to the end: the recording sweep of the
+        // alignment paths uses the same
+        ka.mig_slot[u.item] = int32_t((unsigned(level) << 24) | kMigFinal);
         atomicAdd(&ka.counters->cells[level], cells);
     }
 }
@@ -229,7 +237,8 @@ __device__ __forceinline__ void save_band(const KernelArgs& ka, const DiagArgs& 
 // Loop top, before an odd step, when some unit's band touches its window's
 // outermost slots (every two steps reach one slot further): the window slides by half a virtual lane, or overflows when the band does
 // not fit.
-template <int G, int V, int R>
+// (KEEP = false: an overflowing unit keeps no record)
+template <int G, int V, int R, bool KEEP = true>
 __device__ __forceinline__ void units_slide(const KernelArgs& ka, const DiagArgs& da, DState<V>& u,
                                             int level, int gl, int unit, const Lanes<G>& ln,
                                             uint32_t brink_top, uint32_t brink_bot,
@@ -273,7 +282,15 @@ __device__ __forceinline__ void units_slide(const KernelArgs& ka, const DiagArgs
         u.mt -= by;
         load_planes<G, V, R>(ka, ka.items[u.item], u, gl);
     }
-    if (__any_sync(FULL, ovf)) {
+    if constexpr (!KEEP) {
+        if (ovf) {
+            u.active = false;
+            u.done = true;
+            u.overflow = true;
+#pragma unroll
+            for (int v = 0; v < V; ++v) u.LE[v] = u.LO[v] = 0u;
+        }
+    } else if (__any_sync(FULL, ovf)) {
         int32_t slot = -1;
         if (ovf && gl == 0) slot = mig_alloc(ka, level);
         slot = __shfl_sync(FULL, slot, unit * G);
@@ -328,10 +345,13 @@ __device__ __forceinline__ void unit_maintain(const KernelArgs& ka, const DiagAr
 // One anti-diagonal of every unit of the warp: Q (d-2 on entry) receives d,
 // P holds d-1; inm: the lane's slots inside the matrix.  Returns the warp's vote of lanes with a live slot.  Units without a
 // range compute values without effects.
-template <int G, int V, int R, bool UNIT, bool ODD>
+// REC: rec gets the masks of slots whose value came from the diagonal and, of
+// the others, from the vertical predecessor (meaningful for live slots).
+template <int G, int V, int R, bool UNIT, bool ODD, bool REC>
 __device__ __forceinline__ uint32_t dstep(const DiagArgs& da, DState<V>& u, int at, int gl,
                                           const Lanes<G>& ln, const uint32_t (&inm)[V],
-                                          uint32_t (&Q)[V * R], const uint32_t (&P)[V * R]) {
+                                          uint32_t (&Q)[V * R], const uint32_t (&P)[V * R],
+                                          uint32_t (&rec)[2 * V]) {
     using D = Diag<G, V, R>;
     constexpr int VR = D::VR, C = D::C;
     // the moving operand's codes
@@ -402,46 +422,68 @@ __device__ __forceinline__ uint32_t dstep(const DiagArgs& da, DState<V>& u, int 
         }
         const uint32_t wa6 = wa >> 6, wa12 = wa >> 12, wb6 = wb >> 6, wb12 = wb >> 12;
         uint32_t lk = 0u;
-        uint32_t x[R];
+        SignMask<R> live, from_diag, from_up;
 #pragma unroll
-        for (int h = 0; h < R; ++h) {
-            const int g = v * R + h;
-            // the shifted neighbour, its row code moved by one slot
-            uint32_t sh;
-            if constexpr (ODD) {
-                if (h) {
-                    sh = P[g - 1] - 0x00010001u;
+        for (int j = 0; j < R / 2; ++j) {
+            uint32_t x[2], yd[2], yu[2];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int h = j + half * (R / 2);
+                const int g = v * R + h;
+                // the shifted neighbour, its row code moved by one slot
+                uint32_t sh;
+                if constexpr (ODD) {
+                    if (h) {
+                        sh = P[g - 1] - 0x00010001u;
+                    } else {
+                        const uint32_t lower = v ? P[v * R - 1] : edge;
+                        sh = __byte_perm(lower, P[v * R + R - 1], 0x5432) - 0x00010001u + uint32_t(VR);
+                    }
                 } else {
-                    const uint32_t lower = v ? P[v * R - 1] : edge;
-                    sh = __byte_perm(lower, P[v * R + R - 1], 0x5432) - 0x00010001u + uint32_t(VR);
+                    if (h < R - 1) {
+                        sh = P[g + 1] + 0x00010001u;
+                    } else {
+                        const uint32_t upper = v < V - 1 ? P[(v + 1) * R] : edge;
+                        sh = __byte_perm(P[v * R], upper, 0x5432) + 0x00010001u - (uint32_t(VR) << 16);
+                    }
                 }
-            } else {
-                if (h < R - 1) {
-                    sh = P[g + 1] + 0x00010001u;
+                uint32_t t;
+                if constexpr (UNIT) {
+                    const int q = h & ~1, p = q % 6;  // bits (p, p + 1) of word q / 6
+                    const uint32_t w = (h & 1) ? (q < 6 ? wb : q < 12 ? wb6 : wb12)
+                                               : (q < 6 ? wa : q < 12 ? wa6 : wa12);
+                    t = (w & (0x00030003u << p)) * da.cb[p] + Q[g];
                 } else {
-                    const uint32_t upper = v < V - 1 ? P[(v + 1) * R] : edge;
-                    sh = __byte_perm(P[v * R], upper, 0x5432) + 0x00010001u - (uint32_t(VR) << 16);
+                    const int p = h % 6;
+                    const uint32_t wr = h < 6 ? wa : h < 12 ? wa6 : wa12;
+                    const uint32_t wf = h < 6 ? wb : h < 12 ? wb6 : wb12;
+                    t = (wf & (0x00010001u << p)) * da.cf[p] + Q[g];
+                    t = (wr & (0x00010001u << p)) * da.cb[p] + t;
                 }
+                if constexpr (REC) {
+                    // which predecessor gave the maximum: the diagonal first, then
+                    // the vertical one (keys differ by less than 32768 here)
+                    const uint32_t gap2 = __vimax3_u16x2(P[g], sh, 0u);
+                    yd[half] = t - gap2 + 0x80008000u;
+                    yu[half] = (ODD ? sh - P[g] : P[g] - sh) + 0x80008000u;
+                    Q[g] = __vimax3_u16x2(gap2, t, 0u);
+                } else {
+                    Q[g] = __vimax3_u16x2(P[g], sh, t);
+                }
+                x[half] = Q[g] + thr;
             }
-            uint32_t t;
-            if constexpr (UNIT) {
-                const int q = h & ~1, p = q % 6;  // bits (p, p + 1) of word q / 6
-                const uint32_t w = (h & 1) ? (q < 6 ? wb : q < 12 ? wb6 : wb12)
-                                           : (q < 6 ? wa : q < 12 ? wa6 : wa12);
-                t = (w & (0x00030003u << p)) * da.cb[p] + Q[g];
-            } else {
-                const int p = h % 6;
-                const uint32_t wr = h < 6 ? wa : h < 12 ? wa6 : wa12;
-                const uint32_t wf = h < 6 ? wb : h < 12 ? wb6 : wb12;
-                t = (wf & (0x00010001u << p)) * da.cf[p] + Q[g];
-                t = (wr & (0x00010001u << p)) * da.cb[p] + t;
+            lk = __vimax3_u16x2(lk, Q[v * R + j], Q[v * R + j + R / 2]);
+            live.add(j, x[0], x[1]);
+            if constexpr (REC) {
+                from_diag.add(j, yd[0], yd[1]);
+                from_up.add(j, yu[0], yu[1]);
             }
-            const uint32_t val = __vimax3_u16x2(P[g], sh, t);
-            Q[g] = val;
-            x[h] = val + thr;
-            if (h & 1) lk = __vimax3_u16x2(lk, Q[g - 1], val);
         }
-        L[v] = sign_mask<R>(x) & rb;
+        L[v] = live.get() & rb;
+        if constexpr (REC) {
+            rec[2 * v] = from_diag.get();
+            rec[2 * v + 1] = from_up.get();
+        }
         const uint32_t lkey = max(lk & 0xffffu, lk >> 16);
         // (equal scores: the lower virtual lane's rows come first)
         const bool more = v == 0 || (lkey >> LOG2KS) > (key >> LOG2KS);
@@ -478,6 +520,45 @@ __device__ __forceinline__ uint32_t dstep(const DiagArgs& da, DState<V>& u, int 
     return next_range<G, V, R, ODD>(L, ln, u.rb);
 }
 
+// Slots inside the matrix, rows <= m and columns <= n: step t of the loop body
+// (t odd: an even step) has row m at mt - ceil(t / 2) and the first column at
+// dn + floor(t / 2).
+template <int G, int V, int R>
+__device__ __forceinline__ void matrix_bounds(const DState<V>& u,
+                                              uint32_t (&inm)[Diag<G, V, R>::UNROLL][V]) {
+    using D = Diag<G, V, R>;
+#pragma unroll
+    for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+        for (int v = 0; v < V; ++v) inm[t][v] = FULL;
+    if (__any_sync(FULL, u.mt < D::C + D::UNROLL / 2 || u.dn > -D::UNROLL / 2)) {
+#pragma unroll
+        for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int k0 = __viaddmin_s32_relu(u.dn, t / 2 - v * D::VR, D::VR);
+                const int k1 = __viaddmin_s32_relu(u.mt, 1 - (t + 1) / 2 - v * D::VR, D::VR);
+                inm[t][v] = __funnelshift_lc(~0u, 0u, k1) & ~__funnelshift_lc(~0u, 0u, k0);
+            }
+    }
+}
+
+template <int V>
+__device__ __forceinline__ void state_clear(DState<V>& u) {
+    u.dn = u.mt = 0;
+    u.theta = 32768;
+    u.best = u.bd = u.br = u.X = 0;
+    u.base = u.e = u.phi = 0;
+    u.c32 = 0u;
+    u.cells = u.cells0 = 0ull;
+    u.item = 0u;
+    u.active = u.done = u.overflow = u.migrated = false;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+        u.rb[v] = u.LE[v] = u.LO[v] = u.a0[v] = u.a1[v] = u.b0[v] = u.b1[v] = 0u;
+    u.na0 = u.na1 = u.nb0 = u.nb1 = 0u;
+}
+
 template <int G, int V, int R, bool UNIT>
 __global__ void __launch_bounds__(128, 4)
     k_diag16(KernelArgs ka, DiagArgs da, int level, int queue, int phase) {
@@ -491,18 +572,7 @@ __global__ void __launch_bounds__(128, 4)
 #pragma unroll
     for (int h = 0; h < V * R; ++h) QE[h] = QO[h] = 0u;
     DState<V> u;
-    u.dn = u.mt = 0;
-    u.theta = 32768;
-    u.best = u.bd = u.br = u.X = 0;
-    u.base = u.e = u.phi = 0;
-    u.c32 = 0u;
-    u.cells = u.cells0 = 0ull;
-    u.item = 0u;
-    u.active = u.done = u.overflow = u.migrated = false;
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-        u.rb[v] = u.LE[v] = u.LO[v] = u.a0[v] = u.a1[v] = u.b0[v] = u.b1[v] = 0u;
-    u.na0 = u.na1 = u.nb0 = u.nb1 = 0u;
+    state_clear(u);
     // the outermost slots that the next D::UNROLL steps must find dead
     const uint32_t brink_bot = gl == 0 ? (1u << (D::UNROLL / 2)) - 1u : 0u;
     const uint32_t brink_top = gl == G - 1 ? ((1u << (D::UNROLL / 2)) - 1u) << (D::VR - D::UNROLL / 2) : 0u;
@@ -540,28 +610,133 @@ __global__ void __launch_bounds__(128, 4)
             if (!__any_sync(FULL, u.active || u.done)) break;
         }
         if (__builtin_expect(slide || turn, 0)) next_range<G, V, R, false>(u.LE, ln, u.rb);
-        // slots inside the matrix, rows <= m and columns <= n: step t of the
-        // loop body (t odd: an even step) has row m at mt - ceil(t / 2) and
-        // the first column at dn + floor(t / 2)
         uint32_t inm[D::UNROLL][V];
-#pragma unroll
-        for (int t = 0; t < D::UNROLL; ++t)
-#pragma unroll
-            for (int v = 0; v < V; ++v) inm[t][v] = FULL;
-        if (__any_sync(FULL, u.mt < D::C + D::UNROLL / 2 || u.dn > -D::UNROLL / 2)) {
-#pragma unroll
-            for (int t = 0; t < D::UNROLL; ++t)
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const int k0 = __viaddmin_s32_relu(u.dn, t / 2 - v * D::VR, D::VR);
-                    const int k1 = __viaddmin_s32_relu(u.mt, 1 - (t + 1) / 2 - v * D::VR, D::VR);
-                    inm[t][v] = __funnelshift_lc(~0u, 0u, k1) & ~__funnelshift_lc(~0u, 0u, k0);
-                }
-        }
+        matrix_bounds<G, V, R>(u, inm);
 #pragma unroll
         for (int t = 0; t < D::UNROLL; t += 2) {
-            dstep<G, V, R, UNIT, true>(da, u, t / 2, gl, ln, inm[t], QO, QE);
-            vote = dstep<G, V, R, UNIT, false>(da, u, t / 2, gl, ln, inm[t + 1], QE, QO);
+            uint32_t none[2 * V];
+            dstep<G, V, R, UNIT, true, false>(da, u, t / 2, gl, ln, inm[t], QO, QE, none);
+            vote = dstep<G, V, R, UNIT, false, false>(da, u, t / 2, gl, ln, inm[t + 1], QE, QO, none);
+        }
+        u.e += D::UNROLL / 2;
+        u.dn += D::UNROLL / 2;
+        u.mt -= D::UNROLL / 2;
+        if (--left == 0) {
+            left = iters;
+            unit_maintain<G, V, R>(ka, da, u, gl, QE, QO);
+        }
+    }
+}
+
+// The sweep again, up to each extension's best anti-diagonal, writing for every
+// slot which predecessor its value came from: per lane and loop iteration
+// (UNROLL anti-diagonals) eight words -- one 32-byte sector -- holding, for a
+// virtual lane and anti-diagonal, the mask of slots reached by the diagonal
+// and, of the others, by the vertical move; and per iteration the window's
+// base.  Five instructions more per pair of cells than the extension's sweep.  A
+// band that leaves the window (it fitted one as wide, at other offsets) is
+// flagged for the general sweep.
+template <int G, int V, bool UNIT>
+__global__ void __launch_bounds__(128, V == 1 ? 4 : 3)
+    k_diag16_record(KernelArgs ka, DiagArgs da, DiagRecord rc, int cls) {
+    constexpr int R = 16;
+    using D = Diag<G, V, R>;
+    constexpr unsigned int U = 32 / G;
+    const int lane = threadIdx.x & 31;
+    const int gl = lane % G, unit = lane / G;
+    const Lanes<G> ln(lane);
+    const uint32_t first_item = rc.class_at[cls], n_items = rc.class_at[cls + 1] - first_item;
+    const uint32_t* q = rc.order + first_item;
+    uint32_t QE[V * R], QO[V * R];
+#pragma unroll
+    for (int h = 0; h < V * R; ++h) QE[h] = QO[h] = 0u;
+    DState<V> u;
+    state_clear(u);
+    const uint32_t brink_bot = gl == 0 ? (1u << (D::UNROLL / 2)) - 1u : 0u;
+    const uint32_t brink_top = gl == G - 1 ? ((1u << (D::UNROLL / 2)) - 1u) << (D::VR - D::UNROLL / 2) : 0u;
+    const int iters = da.period / D::UNROLL;
+    int left = iters;
+    bool exhausted = false, first_wave = true;
+    uint4* codes = nullptr;
+    int32_t* bases = nullptr;
+    int dstar = 0;
+    const unsigned int nwarps = gridDim.x * (blockDim.x >> 5);
+    const unsigned int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    for (;;) {
+        if (u.active && 2 * u.e + 1 > dstar) {
+            u.active = false;
+            u.done = true;
+        }
+        const bool slide =
+            __any_sync(FULL, (u.LE[V - 1] & brink_top) != 0u || (u.LE[0] & brink_bot) != 0u);
+        if (__builtin_expect(slide, 0))
+            units_slide<G, V, R, false>(ka, da, u, 0, gl, unit, ln, brink_top, brink_bot, QE, QO);
+        const bool turn = __any_sync(FULL, u.done || (!u.active && !exhausted));
+        if (__builtin_expect(turn, 0)) {
+            if (rc.cells) {
+                int bd, br;
+                unsigned long long cells;
+                unit_totals<G, V>(u, bd, br, cells);
+                if (u.done && !u.overflow && gl == 0) atomicAdd(rc.cells, cells);
+            }
+            if (u.done && u.overflow && gl == 0) {
+                rc.outgrew[u.item] = 1;
+                atomicAdd(rc.n_outgrew, 1u);
+            }
+            if (u.done) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) u.LE[v] = u.LO[v] = 0u;
+            }
+            u.done = false;
+            const bool need = !u.active && !exhausted;
+            const uint32_t want = __ballot_sync(FULL, need && gl == 0);
+            uint32_t id = 0xffffffffu;
+            if (want) {
+                unsigned int slot;
+                if (first_wave) {  // (every unit is idle at the first turn)
+                    slot = gw * U + unsigned(unit);
+                    first_wave = false;
+                } else {
+                    const int leader = __ffs(want) - 1;
+                    unsigned int f = 0u;
+                    if (lane == leader) f = atomicAdd(&rc.next[cls], unsigned(__popc(want)));
+                    f = __shfl_sync(FULL, f, leader);
+                    slot = U * nwarps + f + unsigned(__popc(want & ((1u << (unit * G)) - 1u)));
+                }
+                if (need && slot < n_items) id = q[slot];
+            }
+            if (need) {
+                if (id != 0xffffffffu) {
+                    unit_start<G, V, R, true>(ka, da, u, id, gl, QE, QO);
+                    dstar = rc.dstar[id];
+                    codes = rc.codes + rc.code_off[id] + 2 * gl;
+                    bases = rc.bases + rc.it_off[id];
+                } else {
+                    exhausted = true;
+                }
+            }
+            if (!__any_sync(FULL, u.active)) break;
+        }
+        if (__builtin_expect(slide || turn, 0)) next_range<G, V, R, false>(u.LE, ln, u.rb);
+        uint32_t inm[D::UNROLL][V];
+        matrix_bounds<G, V, R>(u, inm);
+        uint32_t m[D::UNROLL][2 * V];
+#pragma unroll
+        for (int t = 0; t < D::UNROLL; t += 2) {
+            dstep<G, V, R, UNIT, true, true>(da, u, t / 2, gl, ln, inm[t], QO, QE, m[t]);
+            dstep<G, V, R, UNIT, false, true>(da, u, t / 2, gl, ln, inm[t + 1], QE, QO, m[t + 1]);
+        }
+        if (u.active) {
+            const int it = u.e / (D::UNROLL / 2);
+            uint4* c = codes + size_t(it) * (2 * G);
+            if constexpr (V == 1) {
+                c[0] = make_uint4(m[0][0], m[0][1], m[1][0], m[1][1]);
+                c[1] = make_uint4(m[2][0], m[2][1], m[3][0], m[3][1]);
+            } else {
+                c[0] = make_uint4(m[0][0], m[0][1], m[1][0], m[1][1]);
+                c[1] = make_uint4(m[0][2], m[0][3], m[1][2], m[1][3]);
+            }
+            if (gl == 0) bases[it] = u.base;
         }
         u.e += D::UNROLL / 2;
         u.dn += D::UNROLL / 2;
@@ -574,6 +749,18 @@ __global__ void __launch_bounds__(128, 4)
 }
 
 }  // namespace
+
+bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
+    if (!packed_plan(sc, xmax, da)) return false;
+    // the recording sweep subtracts keys: a floor high enough that no two differ
+    // by 32768, and still below every live key
+    const int64_t g = -int64_t(sc.gap), mp = da->mp;
+    const int64_t grow = da->period * g + mp * (da->period / 2 + 1);
+    const int64_t floor = KS * (grow + xmax + mp + 1) + 96;
+    if (floor + KS * (2 * g + 2 * mp + 2) > 32767) return false;
+    da->floor = int(floor);
+    return true;
+}
 
 bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
     const int64_t g = -int64_t(sc.gap), mp = sc.match > 0 ? sc.match : 0;
@@ -614,6 +801,9 @@ bool packed_level(int level) { return level <= 6; }
 // or 4 extensions per warp
 #define LOGAN_PACKED_LATENCY(X) \
     X(0, 1, 32, 2) X(0, 2, 16, 4) X(0, 4, 8, 8) X(1, 1, 32, 4) X(1, 2, 16, 8) X(2, 1, 32, 8)
+
+// class -> (G, V) of its recording sweep
+#define LOGAN_RECORD_CLASSES(X) X(0, 4, 1) X(1, 8, 1) X(2, 16, 1) X(3, 32, 1) X(4, 32, 2)
 
 namespace {
 
@@ -688,6 +878,31 @@ cudaError_t launch_packed_latency(int level, int queue, int units, const KernelA
 #undef CASE
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_record(int cls, const KernelArgs& ka, const DiagArgs& da, const DiagRecord& rc,
+                          int sms, cudaStream_t s) {
+    switch (cls) {
+#define CASE(K, G, V)                                                                            \
+    case K: {                                                                                    \
+        using D = Diag<G, V, 16>;                                                                \
+        static_assert(D::W == level_window(K + 2) && record_lanes(K) == G &&                    \
+                          record_steps(K) == D::UNROLL && (K < 4) == (V == 1),                   \
+                      "class");                                                                  \
+        int n = 0;                                                                               \
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                     \
+            &n, da.unit ? k_diag16_record<G, V, true> : k_diag16_record<G, V, false>, 128, 0);   \
+        if (e != cudaSuccess) return e;                                                          \
+        const int grid = sms * std::max(1, n);                                                   \
+        if (da.unit) k_diag16_record<G, V, true><<<grid, 128, 0, s>>>(ka, da, rc, K);            \
+        else k_diag16_record<G, V, false><<<grid, 128, 0, s>>>(ka, da, rc, K);                   \
+        break;                                                                                   \
+    }
+        LOGAN_RECORD_CLASSES(CASE)
+#undef CASE
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace logan
