@@ -218,7 +218,7 @@ int logan_extend_batch_affine(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
  * Per pair, max(max|entry|, |gap_open| + |gap_extend|) * (m + n) + X must
  * stay below 2^29 (else LOGAN_EINVAL for the pair).  Extensions start in
  * register windows of 64 rows and move to 128, 256 and 512 rows as their
- * bands outgrow them (restarting; with a scalar X the three wider windows
+ * bands outgrow them (restarting; with a scalar X the windows
  * run two cells to a 32-bit register when the matrix's range and X fit
  * 16 bits, LOGAN_OPT_PACKED16 and LOGAN_OPT_MATRIX_PACKED); a band wider
  * than 512 rows, or an X above 2^20 - 4096, continues in one block of 256
@@ -468,18 +468,21 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     the start-level table when X is per pair
                                     or a start level is forced); for the affine
                                     call's windows of 128, 256 and 512 rows
-                                    when 128 * (Xmax + 2*mp + |gap_open| +
-                                    |gap_extend| + 2) + 31 <= 32767 and
-                                    128 * (|mismatch| + |gap_open| +
-                                    2*|gap_extend| + 2*mp + 2) <= 16383;
+                                    and the matrix call's when the like holds
+                                    with the gap extension for |gap| and, o =
+                                    |gap_open|, r = the substitution scores'
+                                    range: 32 * max(D, o + r + 1) + 64 in place
+                                    of 32 * D in the second bound;
                                     otherwise, or with 0, the 32-bit form.
                                     Results are identical either way. */
 #define LOGAN_OPT_AFFINE_PACKED 12 /* read-only: bit l set when affine window
                                     level l (64, 128, 256, 512 rows) ran in
                                     its packed 16-bit form in the context's
                                     last logan_extend_batch_affine call */
-#define LOGAN_OPT_MATRIX_PACKED 13 /* read-only: bit l set when the matrix
-                                    call's window l (64, 128, 256, 512 rows)
+#define LOGAN_OPT_MATRIX_PACKED 13 /* read-only: bit l (l = 1, 2, 3) set when the
+                                    matrix call's window of 128, 256 or 512
+                                    rows (and with them the 64-row one, whose
+                                    bit reads 0)
                                     ran in its packed 16-bit form in the
                                     context's last logan_extend_batch_matrix
                                     call (scalar X only) */

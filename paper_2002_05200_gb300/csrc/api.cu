@@ -73,7 +73,7 @@ struct logan_ctx {
     int blocks_per_sm[kNumLevels] = {};
     int twin_blocks_per_sm[kTwinLevels] = {};
     int affine_blocks_per_sm[4] = {};
-    int affine16_blocks_per_sm[4] = {};
+    int affine16_blocks_per_sm[4][2] = {};  // lanes of 32 slots, of 16 (small batches)
     uint32_t affine_packed_last = 0u;  // bit l: affine level l ran packed in the last call
     uint32_t matrix_packed_last = 0u;  // bit l: matrix window l ran packed in the last call
     // LOGAN_OPT_LONG_ITEM: m + n from which items of levels < kTwinLevels
@@ -360,21 +360,18 @@ PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int3
 }
 
 // Affine levels that run in their packed 16-bit form in this call: those
-// with a packed kernel, when
-//   128 * (Xmax + 2*max(match,0) + |go| + |ge| + 2) + 31 <= 32767  and
-//   128 * (|mismatch| + |go| + 2*|ge| + 2*max(match,0) + 2) <= 16383,
-// Xmax the scalar X, or with per-pair X the upper bound of every X class
-// whose start level is at or below the level.  These bounds keep every
-// 16-bit half inside [0, 65536) through the kernel's additions
-// (xdrop_affine16.cu).
-uint32_t affine16_levels(const logan_ctx* c, Scoring sc, int go, int ge, int32_t X,
-                         const int32_t* Xs, const LevelTable& tab) {
-    if (!c->packed16) return 0u;
+// with a packed kernel whose bounds (diag_affine16.cuh) hold for the scoring
+// and Xmax, the scalar X, or with per-pair X the upper bound of every X class
+// whose start level is at or below the level.
+struct AffinePlan {
+    uint32_t levels = 0u;
+    DiagAffineArgs16 args[4];
+};
+AffinePlan affine16_levels(const logan_ctx* c, Scoring sc, int go, int ge, int32_t X,
+                           const int32_t* Xs, const LevelTable& tab) {
+    AffinePlan pl;
+    if (!c->packed16) return pl;
     static const int64_t upper[kXClasses] = {15, 35, 75, 150, 300, 700, 2000, int64_t(1) << 29};
-    const int64_t mp = std::max<int64_t>(sc.match, 0);
-    const int64_t am = sc.mismatch < 0 ? -int64_t(sc.mismatch) : sc.mismatch;
-    const int64_t ao = -int64_t(go), ae = -int64_t(ge);
-    uint32_t mask = 0u;
     for (int l = 0; l < affine_levels(); ++l) {
         if (!affine16_level(l)) continue;
         int64_t xmax = 0;
@@ -384,12 +381,9 @@ uint32_t affine16_levels(const logan_ctx* c, Scoring sc, int go, int ge, int32_t
             for (int k = 0; k < kXClasses; ++k)
                 if (tab.lv[k] <= l) xmax = std::max(xmax, upper[k]);
         }
-        constexpr int64_t S = 128;  // score scale of the packed keys
-        if (S * (xmax + 2 * mp + ao + ae + 2) + 31 <= 32767 &&
-            S * (am + ao + 2 * ae + 2 * mp + 2) <= 16383)
-            mask |= 1u << l;
+        if (affine16_plan(sc, go, ge, xmax, &pl.args[l])) pl.levels |= 1u << l;
     }
-    return mask;
+    return pl;
 }
 
 // The whole pipeline on `s` (no synchronisation).  plain != 0: one-launch
@@ -446,6 +440,8 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     LevelTable tab = c->table;
     tab.max_level = maxl;
     tab.long_min = long_item_min(c, 2u * n_pairs);
+    AffinePlan aplan;
+    int first_affine = 0;
     if (aff) {
         // affine windows 64 / 128 / 256 / 512 rows by X class, longest first;
         // X too large for the affine keys goes to queue kWarpLevels and is
@@ -453,6 +449,13 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         const int8_t alv[kXClasses] = {0, 0, 1, 1, 2, 3, 3, 3};
         for (int i = 0; i < kXClasses; ++i) tab.lv[i] = alv[i];
         tab.long_min = 0xffffffffu;
+        aplan = affine16_levels(c, sc, aff->open, aff->extend, X, Xs, tab);
+        // a unit of the packed 128-row window costs less than one of the 32-bit
+        // 64-row window: nothing starts below it then
+        if ((aplan.levels >> 1) & 1u) {
+            first_affine = 1;
+            for (int i = 0; i < kXClasses; ++i) tab.lv[i] = std::max<int8_t>(tab.lv[i], 1);
+        }
     }
     int first = 0;
     if (e == cudaSuccess) {
@@ -499,12 +502,15 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     if (aff) {
         // affine levels, narrowest first (each receives the bands that
         // outgrew the previous one), then the rejected items, then combine
-        const uint32_t apacked = affine16_levels(c, sc, aff->open, aff->extend, X, Xs, tab);
+        const uint32_t apacked = aplan.levels;
+        const bool small = n_items <= uint32_t(c->num_sms) * 32u;
         for (int l = 0; l < affine_levels(); ++l) {
             cudaError_t le;
+            if (!((apacked >> l) & 1u) && l < first_affine) continue;  // (nothing starts there)
             if ((apacked >> l) & 1u) {
-                const int grid = c->num_sms * std::max(1, c->affine16_blocks_per_sm[l]);
-                le = launch_affine16_level(l, ka, aff->open, aff->extend, affine_levels(), grid, s);
+                const int grid = c->num_sms * std::max(1, c->affine16_blocks_per_sm[l][small ? 1 : 0]);
+                le = launch_affine16_level(l, ka, aplan.args[l], aff->open, aff->extend,
+                                           affine_levels(), small, grid, s);
             } else {
                 const int grid = c->num_sms * std::max(1, c->affine_blocks_per_sm[l]);
                 le = launch_affine_level(l, ka, aff->open, aff->extend, grid, s);
@@ -807,7 +813,9 @@ int logan_ctx_create(logan_ctx_t** out, int device, const char* autotune_json) {
     for (int l = 0; l < kTwinLevels; ++l) c->twin_blocks_per_sm[l] = twin_blocks_per_sm(l);
     for (int l = 0; l < affine_levels(); ++l) {
         c->affine_blocks_per_sm[l] = affine_blocks_per_sm(l);
-        c->affine16_blocks_per_sm[l] = affine16_level(l) ? affine16_blocks_per_sm(l) : 0;
+        for (int small = 0; small < 2; ++small)
+            c->affine16_blocks_per_sm[l][small] =
+                affine16_level(l) ? affine16_blocks_per_sm(l, small != 0) : 0;
     }
     for (auto& set : c->evs)
         for (auto& ev : set)

@@ -364,6 +364,29 @@ __device__ __forceinline__ void shift_mask(uint32_t (&L)[V], bool on, int gl) {
     }
 }
 
+// Slots inside the matrix, rows <= m and columns <= n: step t of the loop body
+// (t odd: an even step) has row m at mt - ceil(t / 2) and the first column at
+// dn + floor(t / 2).
+template <int G, int V, int R>
+__device__ __forceinline__ void matrix_bounds(const DState<V>& u,
+                                              uint32_t (&inm)[Diag<G, V, R>::UNROLL][V]) {
+    using D = Diag<G, V, R>;
+#pragma unroll
+    for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+        for (int v = 0; v < V; ++v) inm[t][v] = FULL;
+    if (__any_sync(FULL, u.mt < D::C + D::UNROLL / 2 || u.dn > -D::UNROLL / 2)) {
+#pragma unroll
+        for (int t = 0; t < D::UNROLL; ++t)
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int k0 = __viaddmin_s32_relu(u.dn, t / 2 - v * D::VR, D::VR);
+                const int k1 = __viaddmin_s32_relu(u.mt, 1 - (t + 1) / 2 - v * D::VR, D::VR);
+                inm[t][v] = __funnelshift_lc(~0u, 0u, k1) & ~__funnelshift_lc(~0u, 0u, k0);
+            }
+    }
+}
+
 }  // namespace
 
 }  // namespace logan

@@ -138,11 +138,18 @@ int affine_levels();
 int affine_blocks_per_sm(int level);
 cudaError_t launch_affine_level(int level, const KernelArgs& ka, int gap_open, int gap_extend,
                                 int grid, cudaStream_t s);
-// their packed 16-bit forms (xdrop_affine16.cu), for the levels that have one
+// their packed 16-bit forms (xdrop_affine16.cu), for the levels that have one;
+// small: the batch cannot fill the GPU's warps (shorter lanes)
+struct DiagAffineArgs16 {
+    int period, floor;
+};
 bool affine16_level(int level);
-cudaError_t launch_affine16_level(int level, const KernelArgs& ka, int gap_open, int gap_extend,
-                                  int n_levels, int grid, cudaStream_t s);
-int affine16_blocks_per_sm(int level);
+// the constants for this scoring and X, false when the scores do not fit
+bool affine16_plan(Scoring sc, int go, int ge, int64_t xmax, DiagAffineArgs16* out);
+cudaError_t launch_affine16_level(int level, const KernelArgs& ka, const DiagAffineArgs16& plan,
+                                  int gap_open, int gap_extend, int n_levels, bool small, int grid,
+                                  cudaStream_t s);
+int affine16_blocks_per_sm(int level, bool small);
 // bands that outgrow the affine windows, and X too large for their keys:
 // every entry of queue q continues in the device-memory ring kernel
 // (xdrop_matrix.cu) at the workspace ring's width
