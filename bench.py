@@ -838,7 +838,7 @@ def matrix_main(args, rank, world, local):
             # reset, validate A and B, split, four register levels, ring, combine
             "clocks": clk.summary(), "gpu_launches": 10 * args.steps, "cells_per_step": tot,
             "erange_pairs": int((res["status"] == logan.ERANGE).sum()),
-            "roofline": {"bound": "alu", "kernel": "k_mx_group / k_mx16 register windows, then k_mx_ring (whole step)",
+            "roofline": {"bound": "alu", "kernel": "k_diag_affine / k_mx_group register windows, then k_mx_ring (whole step)",
                          "achieved": achieved, "peak": peak, "unit": "Gop/s",
                          "frac": achieved / peak, "traffic": None,
                          "ops_per_cell": OPS_PER_CELL_AFFINE, "cells": cells, "launch_ms": ms,

@@ -259,6 +259,12 @@ int latency_units(const logan_ctx* c, uint32_t n_items, uint32_t long_min) {
     return n_items <= 4u * sms ? 1 : n_items <= 8u * sms ? 2 : 4;
 }
 
+// no more blocks (of four warps) than the batch's items can fill with `units` to a warp
+inline int blocks_for_items(const KernelArgs& ka, int units, int most) {
+    const uint32_t need = (ka.n_items + 4u * uint32_t(units) - 1u) / (4u * uint32_t(units));
+    return int(std::min<uint32_t>(uint32_t(most), std::max(1u, need)));
+}
+
 // The latency form of `level`.  all: it runs every item of the level; else the
 // few long ones, with one block per SM (608 extensions): more blocks, mostly
 // without an item, keep the other forms' blocks from their SMs (20,000 pairs
@@ -268,7 +274,7 @@ int launch_latency(logan_ctx* c, int level, int queue, int units, bool all, cons
                    int phase, cudaStream_t s, const PackedPlan& pk) {
     const int k = units == 4 ? 2 : units - 1;
     const int most = std::max(1, c->latency_blocks_per_sm[level][k]);
-    const int grid = c->num_sms * (all ? most : 1);
+    const int grid = blocks_for_items(ka, units, c->num_sms * (all ? most : 1));
     return launch_packed_latency(level, queue, units, ka, pk.args[level], grid, phase, s) ==
                    cudaSuccess
                ? LOGAN_OK
@@ -281,7 +287,7 @@ int launch_unit(logan_ctx* c, int u, const KernelArgs& ka, int phase, cudaStream
     if (u >= kNumLevels && ((pk.levels >> (u - kNumLevels)) & 1u)) {
         return launch_latency(c, u - kNumLevels, unit_queue(u), units, all, ka, phase, s, pk);
     } else if (u < kNumLevels && ((pk.levels >> u) & 1u)) {
-        const int grid = c->num_sms * std::max(1, c->packed_blocks_per_sm[u]);
+        const int grid = blocks_for_items(ka, 1, c->num_sms * std::max(1, c->packed_blocks_per_sm[u]));
         e = launch_packed_level(u, ka, pk.args[u], grid, phase, s);
     } else if (u >= kNumLevels) {
         const int l = u - kNumLevels;
