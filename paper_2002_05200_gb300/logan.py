@@ -620,6 +620,7 @@ class Server:
     def __init__(self, ctx: Context, budget_bytes: int, max_inflight: int = 4,
                  max_queued: int = 0):
         self._h = ctypes.c_void_p()
+        self._ctx = ctx  # destroying the server writes to its context: it has to live as long
         _check(lib().logan_server_create(ctx._h, int(budget_bytes), int(max_inflight),
                                          int(max_queued), ctypes.byref(self._h)),
                "logan_server_create")
