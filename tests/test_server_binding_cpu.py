@@ -11,7 +11,7 @@ class FakeLib:
     def __getattr__(self, name):
         def call(*args):
             if name.endswith("_create"):
-                args[-1]._obj.value = 1
+                next(a for a in args if hasattr(a, "_obj"))._obj.value = 1
             self.calls.append(name)
             return 0
         return call
