@@ -189,7 +189,9 @@ struct logan_server {
     uint64_t n_done = 0, n_failed = 0, n_cancelled = 0;
     // graphs, timing, concurrent, long item: restored at destroy
     int64_t saved_opts[4] = {0, 0, 1, -2};
-    std::atomic<int> running{0};  // admitted requests not yet completed
+    std::atomic<int> running{0};        // admitted requests not yet completed
+    std::atomic<int64_t> extensions{0};  // and the extensions (two a pair) in them
+    int64_t few_extensions = 0;          // what the GPU runs without queueing, see launch()
 };
 
 namespace {
@@ -218,6 +220,7 @@ void CUDART_CB on_done(void* p) {
             if (q.hbytes) s->harena.release(q.hoff, q.hbytes);
             s->slots[q.slot].ticket = 0;
             s->running.fetch_sub(1);
+            s->extensions.fetch_sub(2 * int64_t(q.r.n_pairs));
             s->n_done++;
         }
     }
@@ -285,12 +288,20 @@ int launch(logan_server* s, uint64_t ticket, Req& q) {
     if (e == cudaSuccess) e = h2d(seeds, r.seeds, size_t(r.n_pairs) * sizeof(logan_seed_t));
     if (e == cudaSuccess && xs) e = h2d(xs, r.X_per_pair, size_t(r.n_pairs) * 4);
     if (e != cudaSuccess) return LOGAN_ECUDA;
-    // long extensions run one to a warp (the step that a request's latency
-    // waits for); with many requests in flight only the longest ones do (more
-    // extensions per instruction for the rest).  A burst of 24 requests of up
-    // to 1,000 uneven pairs: 192 ms with none, 147 ms from 200,000 bases on,
-    // 128 ms from 65,536 on
-    logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, s->running.load() <= 8 ? 65536 : 131072);
+    // long extensions run one to a warp: a request's latency is the longest
+    // one's chain plus, on its one stream, that of the longest of the rest in
+    // the several-to-a-warp forms.  While the extensions in flight do not
+    // queue for the GPU the rest are kept short; a loaded GPU gives only the
+    // longest ones a warp of their own (more extensions per instruction).
+    // Bursts of uneven pairs up to 1 Mbp, from 8,192 / 65,536 / 131,072 bases
+    // on: 24 requests of 33 extensions per SM in all 122-136 / 132-145 /
+    // 142-161 ms, of 142 161-168 / 172-193 / 173-175, 6 requests of 76
+    // 141-142 / 152-153 / 162-169; with eight hardware queues 24 requests of
+    // 33 per SM 184-295 / 220-332 / 255-375
+    const int64_t long_item = s->extensions.load() <= s->few_extensions ? 8192
+                              : s->running.load() <= 8                  ? 65536
+                                                                        : 131072;
+    logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, long_item);
     int rc = logan_extend_batch(s->ctx, &dA, &dB, reinterpret_cast<const logan_seed_t*>(seeds),
                                 r.n_pairs, r.match, r.mismatch, r.gap, r.X,
                                 reinterpret_cast<const int32_t*>(xs), ws, q.ws_bytes,
@@ -342,6 +353,7 @@ void scheduler(logan_server* s) {
             q.t_admit = now_s();
             s->slots[slot].ticket = t;
             s->running.fetch_add(1);
+            s->extensions.fetch_add(2 * int64_t(q.r.n_pairs));
             lk.unlock();
             const int rc = launch(s, t, q);  // q stays valid: entries are erased only when done
             lk.lock();
@@ -358,6 +370,7 @@ void scheduler(logan_server* s) {
                 if (q.hbytes) s->harena.release(q.hoff, q.hbytes);
                 s->slots[slot].ticket = 0;
                 s->running.fetch_sub(1);
+                s->extensions.fetch_sub(2 * int64_t(q.r.n_pairs));
                 s->n_failed++;
                 s->done_cv.notify_all();
             }
@@ -388,6 +401,9 @@ int logan_server_create(logan_ctx_t* ctx, size_t budget_bytes, int max_inflight,
     s->ctx = ctx;
     s->device = int(dev);
     s->max_queued = max_queued ? max_queued : 1u << 20;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
+    s->few_extensions = 160 * int64_t(sms);
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(s->device);
