@@ -565,7 +565,7 @@ int logan_get_escalation(const logan_ctx_t *ctx, int8_t *next, int n);
  * faster with it (step times vary by a few per cent between calls).
  * With the table chosen, the
  * whole sample runs for the two unit forms of each level -- packed 16-bit
- * or 32-bit (LOGAN_OPT_PACKED16 1 / 0) -- crossed with the one-warp rule for
+ * or 32-bit (LOGAN_OPT_PACKED16 1 / 0) -- crossed with the long-item rule for
  * small batches (LOGAN_OPT_LONG_ITEM -2 automatic / -1 several extensions
  * per warp always), and the fastest pair replaces the context's (read back
  * with logan_get_option) when it ran at least 3 % faster.

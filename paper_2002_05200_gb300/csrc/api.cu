@@ -1106,7 +1106,7 @@ int logan_autotune(logan_ctx_t* c, const logan_seqs_t* A, const logan_seqs_t* B,
     c->table = save_table;
     if (rc == LOGAN_OK) rc = set_table(c, chosen, kXClasses);
     // the unit forms with the chosen table: packed 16-bit vs 32-bit, crossed
-    // with the one-warp rule
+    // with the long-item rule
     if (rc == LOGAN_OK) {
         const int64_t forms[4][2] = {{1, -2}, {1, -1}, {0, -2}, {0, -1}};
         float best_ms = -1.f, cur_ms = -1.f;
