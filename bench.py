@@ -628,7 +628,7 @@ def traceback_main(args, b, ctx, stream, rank, world, local, packed):
             "codes": int(ct.sum()), "paths_span_alignments": bool(span_ok),
             "roofline": {
                 "bound": "alu",
-                "kernel": "recording sweep (k_tb_record_warp + k_tb_record_block retries)",
+                "kernel": "recording sweeps (k_diag16_record, k_tb_record_warp/block for the rest)",
                 "achieved": achieved, "peak": peak, "unit": "Gop/s", "frac": achieved / peak,
                 "traffic": None, "ops_per_cell": OPS_PER_CELL, "cells": rec_cells,
                 "launch_ms": mean["record_ms"],
