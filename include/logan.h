@@ -461,8 +461,10 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     linear levels 0-6 when some K in {64, 32, 16,
                                     8, 4} has, with mp = max(match, 0) and
                                     D = K*|gap| + mp*(K/2 + 1),
-                                    32 * (D + Xmax + mp + 1) + 32 <= 32767 and
-                                    32 * (D + 2*|gap| + 2*mp + 2) + 64 <= 32767,
+                                    32 * (D + Xmax + mp + 1) + 32 <= 32767,
+                                    32 * (D + 2*|gap| + 2*mp + 2) + 64 <= 32767
+                                    and 32 * (max(-mismatch, 0) + 2*mp + 2) + 64
+                                    <= 32767,
                                     Xmax the largest X that can reach the level
                                     (the scalar X, or the X-class bounds of
                                     the start-level table when X is per pair

@@ -51,10 +51,7 @@ namespace logan {
 namespace {
 
 constexpr uint32_t FULL = 0xffffffffu;
-constexpr int KS = 32;      // score scale of a key: five bits of row code below it
-constexpr int LOG2KS = 5;
 constexpr int NEGU = -(1 << 20);  // -inf of the 32-bit relative records
-constexpr int kPrefetch = 64;     // steps that the prefetched codes last
 
 // G lanes of V virtual lanes of 2 R slots
 template <int G, int V, int R>

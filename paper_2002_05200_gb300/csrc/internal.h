@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "diag_plan.h"
 #include "logan_dev.cuh"
 
 namespace logan {
@@ -64,21 +65,6 @@ __device__ __forceinline__ int escalate_queue(const KernelArgs& ka, int level, b
     return (twin && nl < kTwinLevels) ? twin_queue(nl) : nl;
 }
 
-// Constants of a packed launch (xdrop_diag16.cu), from the scoring and the
-// largest X that can reach the level.
-struct DiagArgs {
-    int gap;     // gap score per base (<= 0)
-    int mp;      // max(match, 0)
-    int step;    // theta's growth per anti-diagonal: 32 * -gap
-    int floor;   // smallest key (a dead one)
-    int period;  // anti-diagonals between renormalisations (a power of two, 4 .. 64)
-    int unit;    // match 1 and match - mismatch == 2 * (mismatch - 2 gap) (as +1/-1/-1): one
-                 // multiply-add per substitution, a best that grows by 1 at most per anti-diagonal
-    // multipliers of a mask bit at position p: mismatch - 2 gap and match -
-    // mismatch in key units, divided by 2^p
-    uint32_t cb[6], cf[6];
-};
-
 // extension kernels (xdrop_group.cu / xdrop_cta.cu / xdrop_ring.cu)
 cudaError_t launch_warp_level_persistent(int level, const KernelArgs& ka, int grid, int phase,
                                          cudaStream_t s);
@@ -88,7 +74,9 @@ int warp_level_blocks_per_sm(int level);
 // results and band-state records as the level's 32-bit kernel
 bool packed_level(int level);
 // the constants for this scoring and X, false when the scores do not fit
-bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da);
+inline bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
+    return diag_plan(sc.match, sc.mismatch, sc.gap, xmax, da);
+}
 cudaError_t launch_packed_level(int level, const KernelArgs& ka, const DiagArgs& da, int grid,
                                 int phase, cudaStream_t s);
 int packed_level_blocks_per_sm(int level);

@@ -14,6 +14,9 @@
 // by in K steps),
 //     KS * (D + X + mp + 1) + 32        <= 32767   (live keys stay below 65536)
 //     KS * (D + 2 |gap| + 2 mp + 2) + 64 <= 32767  (live keys stay above the floor)
+//     KS * (max(-mismatch, 0) + 2 mp + 2) + 64 <= 32767  (a substitution from a
+//                                       live key stays at or above 0)
+// (diag_plan.h).
 // Then every half-word stays inside [0, 65536) through every addition, and an
 // addition of both halves is one 32-bit operation.
 //
@@ -737,28 +740,6 @@ bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
     if (floor + KS * (2 * g + 2 * mp + 2) > 32767) return false;
     da->floor = int(floor);
     return true;
-}
-
-bool packed_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
-    const int64_t g = -int64_t(sc.gap), mp = sc.match > 0 ? sc.match : 0;
-    for (int period = kPrefetch; period >= 4; period >>= 1) {
-        const int64_t grow = period * g + mp * (period / 2 + 1);
-        if (KS * (grow + xmax + mp + 1) + 32 > 32767 || KS * (grow + 2 * g + 2 * mp + 2) + 64 > 32767)
-            continue;
-        const int base = sc.mismatch - 2 * sc.gap, bonus = sc.match - sc.mismatch;
-        da->gap = sc.gap;
-        da->mp = int(mp);
-        da->step = int(KS * g);
-        da->floor = int(KS * grow + 64);
-        da->period = period;
-        da->unit = bonus == 2 * base && mp == 1 ? 1 : 0;
-        for (int p = 0; p < 6; ++p) {
-            da->cb[p] = uint32_t(base) * uint32_t(KS >> p);
-            da->cf[p] = uint32_t(bonus) * uint32_t(KS >> p);
-        }
-        return true;
-    }
-    return false;
 }
 
 // ---- launches ----
