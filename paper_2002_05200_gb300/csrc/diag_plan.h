@@ -61,4 +61,24 @@ inline bool diag_plan(int match, int mismatch, int gap, int64_t xmax, DiagArgs* 
     return false;
 }
 
+// The constants for the recording sweep, which also subtracts keys: no two that
+// it compares may be 32768 apart.
+//   * The two gap moves' keys: the floor is raised so that no key at or above it
+//     is 32768 above it (and stays below every live key).
+//   * The larger of them, p, against the diagonal's key t.  Where the
+//     substitution is masked t is at or above the floor.  Elsewhere
+//     p - t <= KS (mp - mismatch): a gap move adds nothing to a key, so the cell
+//     above (or left of) a target is at most mp - gap in score above the
+//     target's diagonal predecessor.  diag_plan's third bound gives
+//     KS (mp - mismatch) <= 32767 - 64 - 2 KS.
+inline bool diag_record_plan(int match, int mismatch, int gap, int64_t xmax, DiagArgs* da) {
+    if (!diag_plan(match, mismatch, gap, xmax, da)) return false;
+    const int64_t g = -int64_t(gap), mp = da->mp;
+    const int64_t grow = da->period * g + mp * (da->period / 2 + 1);
+    const int64_t floor = KS * (grow + xmax + mp + 1) + 96;
+    if (floor + KS * (2 * g + 2 * mp + 2) > 32767) return false;
+    da->floor = int(floor);
+    return true;
+}
+
 }  // namespace logan

@@ -110,8 +110,9 @@ struct DiagRecord {
     unsigned int* n_outgrew;
     unsigned long long* cells; // nullable: cells of the completed sweeps
 };
-// (bounds of its keys: packed_plan's, and no two keys 32768 apart)
-bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da);
+inline bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
+    return diag_record_plan(sc.match, sc.mismatch, sc.gap, xmax, da);
+}
 cudaError_t launch_record(int cls, const KernelArgs& ka, const DiagArgs& da, const DiagRecord& rc,
                           int sms, cudaStream_t s);
 // level k's one-warp form (k < kTwinLevels), persistent over twin_queue(k)

@@ -498,14 +498,15 @@ __global__ void __launch_bounds__(128) k_tb_walk_diag(TbArgs t, const uint32_t* 
     const int32_t* bases = t.rec.bases + t.rec.it_off[id];
     int i = x.bi, d = x.bi + x.bj;
     uint32_t cur = 3u, len = 0;
-    int top = -1, lane = -1;  // the loaded lane's iterations top, top - 1, .., top - 15
+    constexpr int kNone = INT_MIN;
+    int top = -1, lane = kNone;  // the loaded lane's iterations top, top - 1, .., top - 15
     int32_t base = 0;         // this thread's iteration: top - me / 2
     uint4 c{};
     while (d > 0) {
         const int it = (d - 1) >> log_steps, st = (d - 1) & ((1 << log_steps) - 1);
         if (it > top || it <= top - 16) {  // (d only falls, so a batch is left downwards)
             top = it;
-            lane = -1;
+            lane = kNone;
             base = top - (me >> 1) >= 0 ? bases[top - (me >> 1)] : 0;
         }
         const int src = 2 * (top - it);
@@ -513,7 +514,11 @@ __global__ void __launch_bounds__(128) k_tb_walk_diag(TbArgs t, const uint32_t* 
         if ((slot >> log_rows) != lane) {
             lane = slot >> log_rows;
             const int mine = top - (me >> 1);
-            if (mine >= 0) c = codes[(size_t(mine) * lanes + lane) * 2 + (me & 1)];
+            // a slot outside the window reads as a diagonal step (it cannot occur on
+            // a walk from a best cell)
+            c = make_uint4(FULL, FULL, FULL, FULL);
+            if (mine >= 0 && lane >= 0 && lane < lanes)
+                c = codes[(size_t(mine) * lanes + lane) * 2 + (me & 1)];
         }
         // two anti-diagonals of a lane per 16 bytes, or a virtual lane's
         const int half = log_steps == 2 ? st >> 1 : (slot >> 5) & 1;

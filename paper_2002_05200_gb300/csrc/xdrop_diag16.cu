@@ -730,18 +730,6 @@ __global__ void __launch_bounds__(128, V == 1 ? 4 : 3)
 
 }  // namespace
 
-bool record_plan(Scoring sc, int64_t xmax, DiagArgs* da) {
-    if (!packed_plan(sc, xmax, da)) return false;
-    // the recording sweep subtracts keys: a floor high enough that no two differ
-    // by 32768, and still below every live key
-    const int64_t g = -int64_t(sc.gap), mp = da->mp;
-    const int64_t grow = da->period * g + mp * (da->period / 2 + 1);
-    const int64_t floor = KS * (grow + xmax + mp + 1) + 96;
-    if (floor + KS * (2 * g + 2 * mp + 2) > 32767) return false;
-    da->floor = int(floor);
-    return true;
-}
-
 // ---- launches ----
 
 // level -> (G, V, R) of its packed form: units of 32-slot lanes, as few as

@@ -21,7 +21,9 @@ int main() {
     while (std::scanf("%d %d %d %lld", &m, &x, &g, &X) == 4) {
         logan::DiagArgs a{};
         const bool ok = logan::diag_plan(m, x, g, X, &a);
-        std::printf("%d %d %d\\n", ok ? 1 : 0, a.period, a.floor);
+        std::printf("%d %d %d ", ok ? 1 : 0, a.period, a.floor);
+        const bool rec = logan::diag_record_plan(m, x, g, X, &a);
+        std::printf("%d %d %d\\n", rec ? 1 : 0, a.period, a.floor);
     }
 }
 """
@@ -64,7 +66,7 @@ def schemes(n):
 def test_no_key_leaves_its_half_word(plan):
     cases = list(schemes(20000))
     taken = far = 0
-    for s, (ok, period, floor) in zip(cases, plan(cases)):
+    for s, (ok, period, floor, *_) in zip(cases, plan(cases)):
         if not ok:
             continue
         lowest, highest, top = key_range(*s, period)
@@ -74,6 +76,22 @@ def test_no_key_leaves_its_half_word(plan):
         taken += 1
         far += max(s[0], 0) - s[1] > 900
     assert taken > 1000 and far > 50
+
+
+def test_recorded_keys_are_less_than_32768_apart(plan):
+    # what the recording sweep subtracts: keys at or above the floor, and a gap
+    # move's key and a live diagonal's, KS (max(match, 0) - mismatch) apart at most
+    cases = list(schemes(20000))
+    taken = 0
+    for s, (*_, ok, period, floor) in zip(cases, plan(cases)):
+        if not ok:
+            continue
+        _, highest, top = key_range(*s, period)
+        assert highest - floor + KS < 32768, s
+        assert floor > top - 32768 and floor < 32768 - KS * (2 * -s[2] + max(s[0], 0)), s
+        assert KS * (max(s[0], 0) - s[1]) + KS < 32768, s
+        taken += 1
+    assert taken > 1000
 
 
 @pytest.mark.parametrize("scheme,ok", [

@@ -1,10 +1,11 @@
 """Scoring schemes at the packed linear kernels' bounds: a mismatch far below two
 gaps on both sides of the bound, and X at the largest value that runs packed.
-Results are integers: every field equals the oracle's."""
+Results are integers: every field, and every path, equals the oracle's."""
 import pytest
 
 from paper_2002_05200_gb300 import logan, synth
 from tests.gpu_common import assert_same, run_gpu, run_oracle
+from tests.test_gpu_traceback import check, gpu_paths
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +38,9 @@ def test_extend(ctx, scheme, long_item):
     b = batch(scheme)
     ctx.set_option(logan.OPT_LONG_ITEM, long_item)
     assert_same(run_gpu(ctx, b, packed2bit=True), run_oracle(b), f"{scheme}")
+
+
+@pytest.mark.parametrize("scheme", SCHEMES)
+def test_paths(ctx, scheme):
+    b = batch(scheme, n_pairs=40)
+    check(b, *gpu_paths(ctx, b, packed2bit=True))
