@@ -354,8 +354,9 @@ PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int3
         } else if (force >= 0) {
             xmax = force <= l ? (Xs ? upper[kXClasses - 1] : X) : 0;
         } else {
+            // (classes above the highest level start at it)
             for (int k = 0; k < kXClasses; ++k)
-                if (tab.lv[k] <= l) xmax = std::max(xmax, upper[k]);
+                if (std::min<int>(tab.lv[k], tab.max_level) <= l) xmax = std::max(xmax, upper[k]);
         }
         if (packed_plan(sc, xmax, &pk.args[l])) pk.levels |= 1u << l;
     }

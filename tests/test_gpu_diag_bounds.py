@@ -1,6 +1,8 @@
 """Scoring schemes at the packed linear kernels' bounds: a mismatch far below two
-gaps on both sides of the bound, and X at the largest value that runs packed.
+gaps on both sides of the bound, X at the largest value that runs packed, and
+X per pair of classes that start at the highest level allowed.
 Results are integers: every field, and every path, equals the oracle's."""
+import numpy as np
 import pytest
 
 from paper_2002_05200_gb300 import logan, synth
@@ -44,3 +46,15 @@ def test_extend(ctx, scheme, long_item):
 def test_paths(ctx, scheme):
     b = batch(scheme, n_pairs=40)
     check(b, *gpu_paths(ctx, b, packed2bit=True))
+
+
+@pytest.mark.parametrize("max_level", [0, 1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("long_item", [0, -1])
+def test_x_classes_above_the_highest_level(ctx, max_level, long_item):
+    # per-pair X: the classes that would start above the highest level start at
+    # it, so its bound has to hold for their X too
+    b = batch((1, -1, -1, 100), n_pairs=72)
+    b.Xs = np.array([10, 60, 140, 400, 1200, 2000], np.int32)[np.arange(72) % 6]
+    ctx.set_option(logan.OPT_MAX_LEVEL, max_level)
+    ctx.set_option(logan.OPT_LONG_ITEM, long_item)
+    assert_same(run_gpu(ctx, b, packed2bit=True), run_oracle(b), f"level {max_level}, long {long_item}")
