@@ -461,16 +461,19 @@ class Context:
         n = ctypes.c_uint64()
         cr = reads.c()
         args = (self._h, ctypes.byref(cr), k, min_freq, max_freq, min_shared)
-        # one call with room for 32 candidates a read (768 B); only a read set
-        # with more runs a second one at the size that the first returned
-        cap = max(1024, 32 * reads.count)
+        # one call with room for 32 candidates a read (96 MiB at most); only a
+        # read set with more runs a second one at the size that the first
+        # returned
+        cap = max(1024, min(32 * reads.count, 1 << 22))
         while True:
             out = torch.empty((cap, 6), dtype=torch.int32, device=f"cuda:{self.device}")
             _check(lib().logan_overlap_candidates(*args, out.data_ptr(), cap, ctypes.byref(n),
                                                   ctypes.c_void_p(stream.cuda_stream)),
                    "logan_overlap_candidates")
             if n.value <= cap:
-                return out[:n.value]
+                # (the call has synchronised; a copy lets a much larger buffer go)
+                out = out[:n.value]
+                return out if 2 * n.value >= cap else out.clone()
             cap = n.value
 
     def overlap_pool(self, reads: DevicePool, stream=None) -> DevicePool:
