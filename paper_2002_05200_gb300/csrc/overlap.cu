@@ -89,16 +89,17 @@ struct ReadIndex {
 
 __global__ void k_read_cells(const uint64_t* __restrict__ first, uint32_t n_reads, uint64_t nk,
                              int shift, uint64_t n_cells, uint32_t* __restrict__ cell) {
-    const uint64_t c = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x;
-    if (c >= n_cells) return;
-    const uint64_t i = min(c << shift, nk - 1);
-    uint32_t lo = 0, hi = n_reads;
-    while (hi - lo > 1u) {
-        const uint32_t mid = lo + ((hi - lo) >> 1);
-        if (first[mid] <= i) lo = mid;
-        else hi = mid;
+    for (uint64_t c = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; c < n_cells;
+         c += uint64_t(gridDim.x) * blockDim.x) {
+        const uint64_t i = min(c << shift, nk - 1);
+        uint32_t lo = 0, hi = n_reads;
+        while (hi - lo > 1u) {
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if (first[mid] <= i) lo = mid;
+            else hi = mid;
+        }
+        cell[c] = lo;
     }
-    cell[c] = lo;
 }
 
 constexpr int kPerThread = 8;
