@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(128) k_tb_walk_diag(TbArgs t, const uint32_t* 
                                                       uint32_t* __restrict__ ops,
                                                       uint64_t* __restrict__ side_n) {
     const int me = int(threadIdx.x & 31u);
-    const uint32_t slot_id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // (a warp per extension: the thread's index passes 32 bits from 2^27 on)
+    const uint64_t slot_id = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (slot_id >= t.rec.class_at[kRecordClasses]) return;
     const uint32_t id = t.rec.order[slot_id];
     const TbItem x = t.info[id], o = t.info[id ^ 1u];
