@@ -330,9 +330,11 @@ int logan_overlap_keep(logan_ctx_t *ctx, const logan_result_t *results,
  * anti-diagonal, recording 2-bit predecessor codes -- in the packed window
  * that its band fitted (up to 2048 rows), else by a warp or a block of 256
  * threads (past 2048 rows in a device-memory ring); a warp or a thread per
- * extension walks back.  The codes take about cells / 8 words of device
- * memory (cells / 16 when that cannot be had) -- meant for the pairs a caller
- * keeps, not whole raw batches.
+ * extension walks back.  The codes take 32 bytes of device memory per
+ * anti-diagonal in a window of 128 rows, 64, 128, 256 and 512 in the wider
+ * ones, and cells / 4 bytes and 16 per anti-diagonal for the general sweeps;
+ * when both cannot be had together every extension takes the general sweep --
+ * meant for the pairs a caller keeps, not whole raw batches.
  * Temporary memory comes stream-ordered from the context's own memory pool,
  * as for logan_overlap_candidates; the call synchronises `stream` (the
  * sweeps run on `stream` and on a second stream the call creates and joins).
@@ -424,6 +426,7 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
  *   LOGAN_OPT_PACKED16      packed 16-bit level kernels (below)
  *   LOGAN_OPT_AFFINE_PACKED which affine levels ran packed (read-only)
  *   LOGAN_OPT_MATRIX_PACKED which matrix windows ran packed (read-only)
+ *   LOGAN_OPT_SCRATCH_MB    size limit of the context's memory pool (below)
  */
 #define LOGAN_OPT_GRAPHS 1
 #define LOGAN_OPT_TIMING 2
@@ -488,6 +491,10 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     ran in its packed 16-bit form in the
                                     context's last logan_extend_batch_matrix
                                     call (scalar X only) */
+#define LOGAN_OPT_SCRATCH_MB 14  /* MiB that the pool which the overlap and
+                                    alignment-path calls take their temporary
+                                    memory from may hold (default 0: no limit
+                                    but the device's); set between calls */
 int logan_set_option(logan_ctx_t *ctx, int option, int64_t value);
 int logan_get_option(const logan_ctx_t *ctx, int option, int64_t *value);
 

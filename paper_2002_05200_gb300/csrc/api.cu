@@ -111,6 +111,7 @@ struct logan_ctx {
     TracebackTiming tb_timing;
     // scratch of the overlap and alignment-path calls (created on first use)
     cudaMemPool_t scratch_pool = nullptr;
+    int64_t scratch_mb = 0;  // its size limit in MiB (0: none)
 };
 
 
@@ -183,6 +184,7 @@ cudaMemPool_t logan::ctx_scratch_pool(logan_ctx_t* c) {
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = c->device;
+        props.maxSize = size_t(c->scratch_mb) << 20;
         cudaMemPool_t p = nullptr;
         if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
         // keep freed scratch mapped between calls: re-mapping gigabytes on
@@ -947,6 +949,13 @@ int logan_set_option(logan_ctx_t* c, int option, int64_t v) {
             c->long_item = v;
             return LOGAN_OK;
         case LOGAN_OPT_PACKED16: c->packed16 = v ? 1 : 0; return LOGAN_OK;
+        case LOGAN_OPT_SCRATCH_MB:
+            if (v < 0 || v > (int64_t(1) << 24)) return LOGAN_EINVAL;
+            // (the next call that needs it makes a new pool)
+            if (c->scratch_pool) cudaMemPoolDestroy(c->scratch_pool);
+            c->scratch_pool = nullptr;
+            c->scratch_mb = v;
+            return LOGAN_OK;
         default: return LOGAN_EINVAL;
     }
 }
@@ -967,6 +976,7 @@ int logan_get_option(const logan_ctx_t* c, int option, int64_t* v) {
         case LOGAN_OPT_PACKED16: *v = c->packed16; return LOGAN_OK;
         case LOGAN_OPT_AFFINE_PACKED: *v = c->affine_packed_last; return LOGAN_OK;
         case LOGAN_OPT_MATRIX_PACKED: *v = c->matrix_packed_last; return LOGAN_OK;
+        case LOGAN_OPT_SCRATCH_MB: *v = c->scratch_mb; return LOGAN_OK;
         default: return LOGAN_EINVAL;
     }
 }

@@ -359,6 +359,7 @@ __global__ void k_tb_general(const Item* __restrict__ items, const ExtRes* __res
     const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= n_items) return;
     TbItem x = info[id];
+    if (x.status == TB_WARP_WIDE) x.status = 0;  // (set by a pass whose storage could not be had)
     const uint64_t dstar = uint64_t(x.bi) + uint64_t(x.bj);
     if (x.wide >= TB_DIAG && !every && !outgrew[id]) {
         item_words[id] = 0u;
@@ -608,19 +609,26 @@ struct TbScratch {
         if (!ok || (pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s)
                          : cudaMallocAsync(&p, bytes, s)) != cudaSuccess) {
             ok = false;
+            (void)cudaGetLastError();  // (reported as LOGAN_ENOMEM, not by the next call)
             return nullptr;
         }
         ptrs.push_back(p);
         return static_cast<T*>(p);
     }
+    // Gives back what was taken since `mark` (a former ptrs.size()), after a
+    // failed request too: what follows can then have that memory.
+    void release(size_t mark) {
+        for (size_t k = mark; k < ptrs.size(); ++k) cudaFreeAsync(ptrs[k], s);
+        ptrs.resize(mark);
+        cudaStreamSynchronize(s);
+        if (pool) cudaMemPoolTrimTo(pool, 0);
+        ok = true;
+    }
     // null instead of failing the call
     template <typename T>
     T* try_get(size_t n) {
         T* p = get<T>(n);
-        if (!p) {
-            ok = true;
-            (void)cudaGetLastError();
-        }
+        if (!p) ok = true;
         return p;
     }
     ~TbScratch() {
@@ -797,9 +805,11 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
     t.info = tinfo;
     t.cells = clk.dcells;
     // The packed sweeps: fixed storage per window slot, about twice what the
-    // general sweep's takes (without room for it, the general sweep takes all).
+    // general sweep's takes.  Without room for it, or for the general sweep of
+    // the rest beside it, it goes back and the general sweep takes all.
     // A second round takes the bands that left their window to the next
     // wider one.
+    const size_t before_rounds = S.ptrs.size();
     struct Round {
         uint64_t *key, *iters, *groups, *it_off, *code_off;
         unsigned int* counts;  // items per class, pop cursors, the number that left their window
@@ -824,7 +834,11 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
         q.order = S.get<uint32_t>(n_items);
         q.outgrew = S.get<int32_t>(n_items);
         q.rec = DiagRecord{};
-        if (!S.ok) return LOGAN_ENOMEM;
+        if (!S.ok && r == 0) return LOGAN_ENOMEM;
+        if (!S.ok) {
+            every = true;
+            break;
+        }
         k_tb_clear<<<(std::max<uint32_t>(n_items, kCounts) + 255) / 256, 256, 0, s>>>(
             q.counts, kCounts, q.outgrew, n_items);
         if (r == 0)
@@ -840,8 +854,11 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
         unsigned int n_class[kRecordClasses + 1] = {};
         if (!tb_scan(S, q.iters, n_items, q.it_off, &total_it) ||
             !tb_scan(S, q.groups, n_items, q.code_off, &total_groups) ||
-            (r == 0 && !tb_scan(S, pc, n_pairs, op_start, &total_codes)))
-            return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
+            (r == 0 && !tb_scan(S, pc, n_pairs, op_start, &total_codes))) {
+            if (S.ok || r == 0) return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
+            every = true;
+            break;
+        }
         if (cudaMemcpyAsync(n_class, q.counts, sizeof(n_class), cudaMemcpyDeviceToHost, s) !=
                 cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
@@ -860,7 +877,11 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
             every = true;
             break;
         }
-        if (!tb_order(S, q.key, n_items, true, q.order)) return S.ok ? LOGAN_ECUDA : LOGAN_ENOMEM;
+        if (!tb_order(S, q.key, n_items, true, q.order)) {
+            if (S.ok) return LOGAN_ECUDA;
+            every = true;
+            break;
+        }
         q.rec = DiagRecord{q.order, q.class_at, q.counts + kRecordClasses + 1, dstar, q.it_off,
                            q.code_off, codes, bases, q.outgrew, q.counts + 2 * kRecordClasses + 1,
                            clk.dcells};
@@ -887,9 +908,17 @@ int run_traceback(int num_sms, const ExtensionViews& v, const logan_seed_t* seed
         if (!n_out) break;
         if (r == 1) rest += n_out;
     }
-    const int32_t* outgrew = rounds[n_rounds ? n_rounds - 1 : 0].outgrew;
-    if (rest || every) {
-        const int rc = run_general(num_sms, v, n_items, sc, ring_log2, every, tinfo, outgrew, t, s, S, clk);
+    if (rest && !every) {
+        const int32_t* outgrew = rounds[n_rounds ? n_rounds - 1 : 0].outgrew;
+        const int rc = run_general(num_sms, v, n_items, sc, ring_log2, false, tinfo, outgrew, t, s, S, clk);
+        if (rc == LOGAN_ENOMEM) every = true;  // (nothing recorded yet)
+        else if (rc != LOGAN_OK) return rc;
+    }
+    if (every) {
+        S.release(before_rounds);
+        if (clk.dcells) cudaMemsetAsync(clk.dcells, 0, sizeof(unsigned long long), s);
+        clk.words = 0;
+        const int rc = run_general(num_sms, v, n_items, sc, ring_log2, true, tinfo, nullptr, t, s, S, clk);
         if (rc != LOGAN_OK) return rc;
     }
     clk.mark(TbClock::REC_END, s);
