@@ -295,7 +295,12 @@ __device__ __forceinline__ void units_slide(const KernelArgs& ka, const DiagArgs
         }
     } else if (__any_sync(FULL, ovf)) {
         int32_t slot = -1;
-        if (ovf && gl == 0) slot = mig_alloc(ka, level);
+        if (ovf && gl == 0) {
+            // (an extension that moved to a window as wide writes over its own record)
+            const int pool = mig_pool_level(level, D::W);
+            const int32_t own = ka.mig_slot[u.item];
+            slot = own >= 0 && (own >> 24) == pool ? own : mig_alloc(ka, pool);
+        }
         slot = __shfl_sync(FULL, slot, unit * G);
         // first and last live slots, the best cell, the cells
         int lo = D::W, hi = -1, bd, br;
@@ -818,7 +823,8 @@ cudaError_t launch_packed_latency(int level, int queue, int units, const KernelA
     switch (latency_form(level, units)) {
 #define CASE(K, U, G, R)                                                                  \
     case 10 * K + U:                                                                      \
-        static_assert(Diag<G, 1, R>::W == level_window(K + 2) && 32 / G == U, "window"); \
+        static_assert(Diag<G, 1, R>::W == level_window(K + 2) && 32 / G == U &&          \
+                          Diag<G, 1, R>::W <= mig_rows(K + 2), "window and record");      \
         return launch<G, 1, R>(level, queue, ka, da, grid, phase, s);
         LOGAN_PACKED_LATENCY(CASE)
 #undef CASE
