@@ -191,13 +191,9 @@ enum MigField {
 constexpr int MIG_RELATIVE = 1;
 constexpr int MIG_ABSOLUTE = 2;
 // rows of a level's record: its window, or the 64 slots that level 0 runs packed
+// (the 128-slot latency forms of levels 0 and 1 use level 2's records)
 __host__ __device__ constexpr int mig_rows(int level) {
     return level_window(level) < 64 ? 64 : level_window(level);
-}
-// the level whose pool takes the records of `level`'s form with a window of w rows
-// (the latency forms of levels 0 and 1 hold 128 rows, as level 2)
-__host__ __device__ constexpr int mig_pool_level(int level, int w) {
-    return w <= mig_rows(level) ? level : 2;
 }
 __host__ __device__ constexpr int mig_stride(int level) { return kMigHeader + 2 * mig_rows(level); }
 

@@ -296,10 +296,15 @@ __device__ __forceinline__ void units_slide(const KernelArgs& ka, const DiagArgs
     } else if (__any_sync(FULL, ovf)) {
         int32_t slot = -1;
         if (ovf && gl == 0) {
-            // (an extension that moved to a window as wide writes over its own record)
-            const int pool = mig_pool_level(level, D::W);
-            const int32_t own = ka.mig_slot[u.item];
-            slot = own >= 0 && (own >> 24) == pool ? own : mig_alloc(ka, pool);
+            if constexpr (R < 16 && D::W == level_window(2)) {
+                // the 128-slot latency forms of levels 0-2 share a pool: an extension
+                // that moves among them writes over its own record
+                constexpr int pool = 2;
+                const int32_t own = ka.mig_slot[u.item];
+                slot = own >= 0 && (own >> 24) == pool ? own : mig_alloc(ka, pool);
+            } else {
+                slot = mig_alloc(ka, level);
+            }
         }
         slot = __shfl_sync(FULL, slot, unit * G);
         // first and last live slots, the best cell, the cells
