@@ -267,6 +267,14 @@ inline int blocks_for_items(const KernelArgs& ka, int units, int most) {
     return int(std::min<uint32_t>(uint32_t(most), std::max(1u, need)));
 }
 
+// Items of a level that take its packed latency form beside the others, at most:
+// two for each of the four warps per SM that the launch below has.  With more the
+// longest stay (whole length buckets) and the rest run several to a warp:
+// 3,000 pairs of 200 kbp, all long, took 266 ms four to an SM and take 62 several to a
+// warp (32-bit latency form with the whole GPU: 194); 1,216 extensions of
+// one length are about even.
+constexpr uint32_t kLongItemsPerSm = 8;
+
 // The latency form of `level`.  all: it runs every item of the level; else the
 // few long ones, with one block per SM (608 extensions): more blocks, mostly
 // without an item, keep the other forms' blocks from their SMs (20,000 pairs
@@ -449,6 +457,12 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     LevelTable tab = c->table;
     tab.max_level = maxl;
     tab.long_min = long_item_min(c, 2u * n_pairs);
+    const int64_t forced = c->force_level >= 0 ? std::min<int64_t>(c->force_level, maxl) : -1;
+    const PackedPlan packed =
+        (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced);
+    // (every item in latency form has the whole GPU, the 32-bit forms do in any case)
+    tab.capped = tab.long_min == 0u ? 0u : packed.levels;
+    tab.long_cap = kLongItemsPerSm * uint32_t(c->num_sms);
     AffinePlan aplan;
     int first_affine = 0;
     if (aff) {
@@ -505,9 +519,6 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         ka.mig_pool[l] = L.mig_cap[l] ? reinterpret_cast<int32_t*>(ws + L.mig_pool[l]) : nullptr;
     }
     ka.mig_slot = reinterpret_cast<int32_t*>(ws + L.mig_slot);
-    const int64_t forced = c->force_level >= 0 ? std::min<int64_t>(c->force_level, maxl) : -1;
-    const PackedPlan packed =
-        (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced);
     if (aff) {
         // affine levels, narrowest first (each receives the bands that
         // outgrew the previous one), then the rejected items, then combine

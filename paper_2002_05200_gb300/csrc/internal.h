@@ -169,8 +169,10 @@ struct LevelTable {
     int8_t lv[8];
     int max_level;
     // items with m + n >= long_min that start below level kTwinLevels go to
-    // that level's one-warp form (0xffffffff: none)
+    // that level's one-warp form (0xffffffff: none); of the levels in `capped`
+    // (bit l: level l) only the longest long_cap at most do
     uint32_t long_min;
+    uint32_t long_cap, capped;
 };
 cudaError_t launch_bin(const Item* items, uint32_t n_items, LevelTable table, int force_level, uint32_t* hist, uint32_t* queues, uint32_t qcap,
                        Counters* counters, cudaStream_t s);

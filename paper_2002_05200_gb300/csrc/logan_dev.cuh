@@ -107,6 +107,7 @@ struct Counters {
     unsigned int head2[kQueues];               // pop cursor of the escalated entries
     unsigned int n_long[kNumLevels];           // binned entries for the latency form (the first ones)
     unsigned int head_long[kNumLevels];        // their pop cursor
+    unsigned int long_buckets[kTwinLevels];    // length buckets whose long items take the latency form
 };
 
 // Which entries of a level's queue a launch processes: the binned (initial)

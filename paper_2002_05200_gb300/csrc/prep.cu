@@ -192,32 +192,68 @@ __global__ void k_bin_hist(const Item* __restrict__ items, uint32_t n, LevelTabl
 // fallback ring's queue gets no binned items)
 constexpr int kScanThreads = 32 * kQueues;
 static_assert(kBuckets == 128, "four buckets per lane");
+// A level's long items past table.long_cap, whole buckets of the shorter ones,
+// go back to the level's own queue.
 __global__ void __launch_bounds__(kScanThreads)
-    k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c, uint32_t long_min) {
+    k_bin_scan(uint32_t* __restrict__ hist, Counters* __restrict__ c, LevelTable table) {
     const int lane = threadIdx.x & 31, l = threadIdx.x >> 5, t = threadIdx.x;
-    uint4 v = reinterpret_cast<const uint4*>(hist + l * kBuckets)[lane];
-    const uint32_t sum = v.x + v.y + v.z + v.w;
-    uint32_t incl = sum;
+    const uint32_t long_min = table.long_min;
+    // inclusive prefixes of four buckets per lane over the warp
+    auto prefix = [lane](const uint32_t (&x)[4], uint32_t (&incl)[4]) {
+        const uint32_t sum = x[0] + x[1] + x[2] + x[3];
+        uint32_t at = sum;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
+        }
+        at -= sum;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) incl[i] = at += x[i];
+    };
+    const uint4 v4 = reinterpret_cast<const uint4*>(hist + l * kBuckets)[lane];
+    uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w}, incl[4];
+    const int lv = l < kTwinLevels ? l : l > kNumLevels ? l - twin_queue(0) : -1;
+    const bool capped = lv >= 0 && ((table.capped >> lv) & 1u);
+    uint4 w4 = v4;  // the level's long items
+    if (capped && l < kTwinLevels)
+        w4 = reinterpret_cast<const uint4*>(hist + twin_queue(l) * kBuckets)[lane];
+    __syncthreads();  // (each is read by its own warp and its level's, then overwritten)
+    if (capped) {
+        const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+        uint32_t kept = 0u;
+        prefix(w, incl);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool keep = incl[i] <= table.long_cap;
+            kept += keep ? 1u : 0u;
+            if (l < kTwinLevels) v[i] += keep ? 0u : w[i];
+            else v[i] = keep ? v[i] : 0u;
+        }
+        kept = __reduce_add_sync(0xffffffffu, kept);
+        if (l < kTwinLevels && lane == 0) c->long_buckets[l] = kept;
+    } else if (l < kTwinLevels && lane == 0) {
+        c->long_buckets[l] = kBuckets;
     }
-    const uint32_t at = incl - sum;  // exclusive prefixes = cursors
-    const uint4 e = make_uint4(at, at + v.x, at + v.x + v.y, at + v.x + v.y + v.z);
-    reinterpret_cast<uint4*>(hist + l * kBuckets)[lane] = e;
-    // buckets that hold only items of m + n >= long_min come first
-    const int n_long_buckets = long_min == 0u            ? kBuckets
-                               : long_min == 0xffffffffu ? 0
-                                                         : kBuckets - 1 - work_bucket(long_min - 1u, 0u);
+    prefix(v, incl);
+    reinterpret_cast<uint4*>(hist + l * kBuckets)[lane] =
+        make_uint4(incl[0] - v[0], incl[1] - v[1], incl[2] - v[2], incl[3] - v[3]);  // cursors
     if (lane == 31) {
-        c->tail[l] = incl;
-        c->started[l] = incl;
-        if (l < kNumLevels && n_long_buckets == kBuckets) c->n_long[l] = incl;
+        c->tail[l] = incl[3];
+        c->started[l] = incl[3];
     }
-    if (l < kNumLevels && n_long_buckets < kBuckets && lane == n_long_buckets / 4) {
-        const uint32_t p[4] = {e.x, e.y, e.z, e.w};
-        c->n_long[l] = p[n_long_buckets & 3];
+    // buckets that hold only items of m + n >= long_min come first
+    if (l < kNumLevels) {
+        const int n_long_buckets = long_min == 0u            ? kBuckets
+                                   : long_min == 0xffffffffu ? 0
+                                                             : kBuckets - 1 - work_bucket(long_min - 1u, 0u);
+        const uint32_t cap = ((table.capped >> l) & 1u) ? table.long_cap : 0xffffffffu;
+        uint32_t n = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (4 * lane + i < n_long_buckets && incl[i] <= cap) n = incl[i];
+        n = __reduce_max_sync(0xffffffffu, n);
+        if (lane == 0) c->n_long[l] = n;
     }
     if (t < kQueues) {
         c->head[t] = 0u;
@@ -232,13 +268,16 @@ __global__ void __launch_bounds__(kScanThreads)
 
 __global__ void k_bin_scatter(const Item* __restrict__ items, uint32_t n, LevelTable table,
                               int force, int maxl, uint32_t* __restrict__ cursor,
-                              uint32_t* __restrict__ queues, uint32_t qcap) {
+                              const Counters* __restrict__ c, uint32_t* __restrict__ queues,
+                              uint32_t qcap) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const Item it = items[i];
     if (it.flags & ITEM_SKIP) return;
-    const int q = item_queue(it, table, force, maxl);
-    const uint32_t pos = atomicAdd(&cursor[q * kBuckets + (kBuckets - 1 - work_bucket(it.m, it.n))], 1u);
+    int q = item_queue(it, table, force, maxl);
+    const int bucket = kBuckets - 1 - work_bucket(it.m, it.n);
+    if (q > kNumLevels && bucket >= int(c->long_buckets[q - twin_queue(0)])) q -= twin_queue(0);
+    const uint32_t pos = atomicAdd(&cursor[q * kBuckets + bucket], 1u);
     queues[size_t(q) * qcap + pos] = i;
 }
 
@@ -331,10 +370,10 @@ cudaError_t launch_bin(const Item* items, uint32_t n_items, LevelTable table, in
         const unsigned int g = min(blocks_for(n_items, 256), 1024u);
         k_bin_hist<<<g, 256, 0, s>>>(items, n_items, table, force_level, maxl, hist);
     }
-    k_bin_scan<<<1, kScanThreads, 0, s>>>(hist, counters, table.long_min);
+    k_bin_scan<<<1, kScanThreads, 0, s>>>(hist, counters, table);
     if (n_items)
         k_bin_scatter<<<blocks_for(n_items, 256), 256, 0, s>>>(items, n_items, table, force_level,
-                                                               maxl, hist, queues, qcap);
+                                                               maxl, hist, counters, queues, qcap);
     return cudaGetLastError();
 }
 
