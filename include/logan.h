@@ -455,8 +455,10 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     m + n >= v; -1: never; -2 (default):
                                     automatic -- every item when the batch
                                     has at most 32 items per SM, else
-                                    m + n >= 131072.  Results never depend on
-                                    it. */
+                                    m + n >= 131072.  Where only some items
+                                    take it, at most 8 per SM of a packed
+                                    level do, the longest.  Results never
+                                    depend on it. */
 #define LOGAN_OPT_PACKED16 11    /* 1 (default): a window level that has a
                                     packed form (two 16-bit cells per 32-bit
                                     register) runs it when the call's scoring
