@@ -616,8 +616,10 @@ int logan_autotune_save(const logan_ctx_t *ctx, const char *path);
  * waits for that request's copies); so is a request whose host buffers are
  * all pinned.  The server uses the context exclusively (graphs, timing and
  * concurrent levels off: each request runs on its slot's stream;
- * LOGAN_OPT_LONG_ITEM set per request: 65536 while at most 8 requests are
- * in flight, else 131072) until logan_server_destroy, which restores those
+ * LOGAN_OPT_LONG_ITEM set per request: 8192 while the extensions in flight
+ * are at most 160 per SM, else 65536 while at most 8 requests are in flight,
+ * else 131072; a level's latency form takes at most the request's share of
+ * 32 extensions per SM) until logan_server_destroy, which restores those
  * four options; do not call other functions on that context
  * meanwhile.  The slots overlap only as far as the device's hardware work
  * queues allow: set CUDA_DEVICE_MAX_CONNECTIONS (up to 32) to at least

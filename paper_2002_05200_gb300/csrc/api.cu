@@ -79,6 +79,7 @@ struct logan_ctx {
     // LOGAN_OPT_LONG_ITEM: m + n from which items of levels < kTwinLevels
     // take the latency form; -1 never, -2 automatic
     int64_t long_item = -2;
+    uint32_t long_cap = 0xffffffffu;  // and how many of them per level, see ctx_set_long_cap
     // LOGAN_OPT_PACKED16: 1 = run a level in its packed 16-bit form when the
     // call's scoring and X provably fit (see packed16_levels), 0 = never
     int64_t packed16 = 1;
@@ -177,6 +178,8 @@ Layout make_layout(const logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t
 TracebackTiming* logan::ctx_traceback_timing(logan_ctx_t* c) { return &c->tb_timing; }
 
 void logan::ctx_set_matrix_packed(logan_ctx_t* c, uint32_t levels) { c->matrix_packed_last = levels; }
+
+void logan::ctx_set_long_cap(logan_ctx_t* c, uint32_t items) { c->long_cap = items; }
 
 cudaMemPool_t logan::ctx_scratch_pool(logan_ctx_t* c) {
     if (!c->scratch_pool) {
@@ -462,7 +465,7 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced);
     // (every item in latency form has the whole GPU, the 32-bit forms do in any case)
     tab.capped = tab.long_min == 0u ? 0u : packed.levels;
-    tab.long_cap = kLongItemsPerSm * uint32_t(c->num_sms);
+    tab.long_cap = std::min(kLongItemsPerSm * uint32_t(c->num_sms), c->long_cap);
     AffinePlan aplan;
     int first_affine = 0;
     if (aff) {

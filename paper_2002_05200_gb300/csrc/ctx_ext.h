@@ -26,6 +26,11 @@ cudaMemPool_t ctx_scratch_pool(logan_ctx_t* c);
 // LOGAN_OPT_MATRIX_PACKED)
 void ctx_set_matrix_packed(logan_ctx_t* c, uint32_t levels);
 
+// At most this many items of a level take its packed latency form beside the
+// other forms (0xffffffff: what one call alone may).  The server's, which
+// knows what else is in flight.
+void ctx_set_long_cap(logan_ctx_t* c, uint32_t items);
+
 // Device views into the workspace of a finished logan_extend_batch call
 // with the same pools and pair count: the 2-bit words of both pools, the
 // split items (two per pair, left first), every item's result (best cell,

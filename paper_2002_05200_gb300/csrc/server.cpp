@@ -41,6 +41,10 @@
 
 #include "../../include/logan.h"
 
+namespace logan {
+void ctx_set_long_cap(logan_ctx_t* c, uint32_t items);  // (ctx_ext.h, which needs CUDA)
+}
+
 namespace {
 
 constexpr size_t kAlign = 256;
@@ -192,6 +196,7 @@ struct logan_server {
     std::atomic<int> running{0};        // admitted requests not yet completed
     std::atomic<int64_t> extensions{0};  // and the extensions (two a pair) in them
     int64_t few_extensions = 0;          // what the GPU runs without queueing, see launch()
+    int64_t latency_extensions = 0;      // what it runs in latency forms at once
 };
 
 namespace {
@@ -302,6 +307,12 @@ int launch(logan_server* s, uint64_t ticket, Req& q) {
                               : s->running.load() <= 8                  ? 65536
                                                                         : 131072;
     logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, long_item);
+    // The requests in flight share the GPU's warps: each one's latency forms get
+    // its share of two extensions a warp (16 requests of 400 pairs of 10 kbp, all
+    // long: 16.2 ms without this, 9.9 with it, 11.0 in 32 bits several to a warp)
+    const int64_t share = s->latency_extensions * 2 * int64_t(r.n_pairs) /
+                          std::max<int64_t>(s->extensions.load(), 2 * int64_t(r.n_pairs));
+    logan::ctx_set_long_cap(s->ctx, uint32_t(share));
     int rc = logan_extend_batch(s->ctx, &dA, &dB, reinterpret_cast<const logan_seed_t*>(seeds),
                                 r.n_pairs, r.match, r.mismatch, r.gap, r.X,
                                 reinterpret_cast<const int32_t*>(xs), ws, q.ws_bytes,
@@ -404,6 +415,7 @@ int logan_server_create(logan_ctx_t* ctx, size_t budget_bytes, int max_inflight,
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
     s->few_extensions = 160 * int64_t(sms);
+    s->latency_extensions = 32 * int64_t(sms);  // four blocks of four warps per SM, two each
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(s->device);
@@ -581,6 +593,7 @@ int logan_server_destroy(logan_server_t* s) {
     logan_set_option(s->ctx, LOGAN_OPT_TIMING, s->saved_opts[1]);
     logan_set_option(s->ctx, LOGAN_OPT_CONCURRENT, s->saved_opts[2]);
     logan_set_option(s->ctx, LOGAN_OPT_LONG_ITEM, s->saved_opts[3]);
+    logan::ctx_set_long_cap(s->ctx, 0xffffffffu);
     delete s;
     return LOGAN_OK;
 }

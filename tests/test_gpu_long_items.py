@@ -66,3 +66,23 @@ def test_many_long_extensions(ctx):
             best = min(best, t0.elapsed_time(t1))
         return best
     assert ms(-2) < 2 * ms(-1)
+
+
+def test_requests_share_the_latency_forms(ctx):
+    # more long extensions in one request than its latency forms take, then in
+    # six requests together
+    b = synth.uniform_pairs(n_pairs=64, length=9000, X=50, seed=8)
+    ref = run_oracle(b)
+    take = np.arange(700) % 64
+    b.seeds = b.seeds[take]
+    srv = logan.Server(ctx, 8 << 30, 8)
+    try:
+        for n in (1, 6):
+            reqs = [logan.HostRequest(b) for _ in range(n)]
+            for t in [srv.submit(r) for r in reqs]:
+                assert srv.wait(t)[0] == logan.OK
+            for r in reqs:
+                got = r.results.numpy().view(logan.RESULT_DTYPE).reshape(-1)
+                assert_same(got, ref[take], f"{n} requests")
+    finally:
+        srv.close()
