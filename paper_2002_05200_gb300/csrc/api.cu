@@ -47,7 +47,7 @@ struct AuxSet {
 // the levels that run packed in a call (bit l: level l) and their constants
 struct PackedPlan {
     uint32_t levels = 0u;
-    DiagArgs args[kNumLevels];
+    DiagArgs args[kNumLevels] = {};
 };
 inline size_t up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -253,15 +253,28 @@ void default_table(LevelTable& t) {
     t.max_level = kNumLevels - 1;
 }
 
-// Extensions per warp of a packed latency form.  Few items (or the long ones
-// of a batch): one, the shortest step.  A small batch with more items than
-// four warps per SM would queue for the schedulers with one per warp: two or
-// four share a warp's step (16 pairs of 2 kbp: 0.28 / 0.32 / 0.40 ms with 1 / 2 / 4
-// per warp; 1,000 pairs: 0.57 / 0.53 / 0.50 ms).
-int latency_units(const logan_ctx* c, uint32_t n_items, uint32_t long_min) {
-    if (long_min != 0u) return 1;
-    const uint32_t sms = uint32_t(c->num_sms);
-    return n_items <= 4u * sms ? 1 : n_items <= 8u * sms ? 2 : 4;
+// Extensions per warp of a level's packed latency form when every item of a small
+// batch takes it (`all`; the long ones of a larger batch: one, the shortest
+// step), by the items per SM.  Few items: one to a warp.  More warps than the
+// schedulers issue in turn lengthen every step, two or four extensions share one
+// then.  unit: the substitution is one multiply-add and the best a vote (+1 / -1 /
+// -1); else a step costs more issue slots, in two and four to a warp most of
+// all.  Pairs of 3 kbp, one / two / four to a warp, ms:
+//     per SM            8.6                 13.2                 19.7
+//     +1/-1/-1, X=60    .76  .69  .70       .95  .70  .70        1.14  .89  .87
+//       lognormal       2.37 2.35 2.56      2.53 2.35 2.52       2.47 2.64 2.67
+//     +2/-3/-5, X=60    .81  .79  .85       1.01 .80  .85        1.22  .99  1.01
+//       lognormal       1.36 1.53 1.83      1.63 1.56 1.83       1.58 1.81 1.96
+// (the 32-bit one-warp forms: 1.07, 3.40, 1.06, 1.64; 1.34, 3.60, 1.34, 1.81; 1.90,
+// 4.25, 1.88, 2.44).  The 256-slot form (level 3) has two to a warp at most; levels 0
+// and 1 have four with half the window (xdrop_diag16.cu) when not unit.
+int latency_units(const logan_ctx* c, int level, uint32_t n_items, bool all, bool unit) {
+    if (!all || level > 3) return 1;
+    const uint32_t per_sm = (n_items + uint32_t(c->num_sms) - 1u) / uint32_t(c->num_sms);
+    if (level == 3) return unit ? (per_sm <= 4u ? 1 : per_sm <= 8u ? 2 : 4) : per_sm <= 24u ? 1 : 4;
+    if (unit) return per_sm <= 4u ? 1 : per_sm <= 16u ? 2 : 4;
+    if (level <= 1) return per_sm <= (level == 0 ? 12u : 8u) ? 1 : 4;
+    return per_sm <= 12u ? 1 : per_sm <= 24u ? 2 : 4;
 }
 
 // no more blocks (of four warps) than the batch's items can fill with `units` to a warp
@@ -283,8 +296,9 @@ constexpr uint32_t kLongItemsPerSm = 8;
 // without an item, keep the other forms' blocks from their SMs (20,000 pairs
 // of 5 kbp, none long: 7.1 ms with three, 6.8 with one; uneven pairs
 // up to 1 Mbp 236 and 227 ms).
-int launch_latency(logan_ctx* c, int level, int queue, int units, bool all, const KernelArgs& ka,
-                   int phase, cudaStream_t s, const PackedPlan& pk) {
+int launch_latency(logan_ctx* c, int level, int queue, bool all, const KernelArgs& ka, int phase,
+                   cudaStream_t s, const PackedPlan& pk) {
+    const int units = latency_units(c, level, ka.n_items, all, pk.args[level].unit != 0);
     const int k = units == 4 ? 2 : units - 1;
     const int most = std::max(1, c->latency_blocks_per_sm[level][k]);
     const int grid = blocks_for_items(ka, units, c->num_sms * (all ? most : 1));
@@ -295,10 +309,10 @@ int launch_latency(logan_ctx* c, int level, int queue, int units, bool all, cons
 }
 
 int launch_unit(logan_ctx* c, int u, const KernelArgs& ka, int phase, cudaStream_t s,
-                const PackedPlan& pk, int units, bool all) {
+                const PackedPlan& pk, bool all) {
     cudaError_t e;
     if (u >= kNumLevels && ((pk.levels >> (u - kNumLevels)) & 1u)) {
-        return launch_latency(c, u - kNumLevels, unit_queue(u), units, all, ka, phase, s, pk);
+        return launch_latency(c, u - kNumLevels, unit_queue(u), all, ka, phase, s, pk);
     } else if (u < kNumLevels && ((pk.levels >> u) & 1u)) {
         const int grid = blocks_for_items(ka, 1, c->num_sms * std::max(1, c->packed_blocks_per_sm[u]));
         e = launch_packed_level(u, ka, pk.args[u], grid, phase, s);
@@ -566,7 +580,6 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         first_escalated = l + 1;
     }
     const bool all = tab.long_min == 0u;  // every item takes its level's latency form
-    const int units = latency_units(c, n_items, tab.long_min);
     uint32_t p1_levels = 0, p2_levels = 0;
     cudaEvent_t* ev = c->ev;
     auto rec = [&](int idx, cudaStream_t st) {
@@ -600,14 +613,14 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
                 // the long items of the 512-row level in its latency form, beside the rest
                 cudaStream_t sl = ax ? ax->st[kUnits] : s;
                 if (ax && cudaStreamWaitEvent(sl, ax->fork, 0) != cudaSuccess) return LOGAN_ECUDA;
-                if (launch_latency(c, u, u, 1, all, ka, PHASE_LONG, sl, packed) != LOGAN_OK)
+                if (launch_latency(c, u, u, all, ka, PHASE_LONG, sl, packed) != LOGAN_OK)
                     return LOGAN_ECUDA;
                 if (ax && cudaEventRecord(ax->join[kUnits], sl) != cudaSuccess) return LOGAN_ECUDA;
                 phase = PHASE_REST;
                 ++launches;
             }
             if (!(phase == PHASE_REST && tab.long_min == 0u) &&
-                launch_unit(c, u, ka, phase, st, packed, units, all) != LOGAN_OK)
+                launch_unit(c, u, ka, phase, st, packed, all) != LOGAN_OK)
                 return LOGAN_ECUDA;
             if (phase == PHASE_REST && ax &&
                 cudaStreamWaitEvent(st, ax->join[kUnits], 0) != cudaSuccess)
@@ -629,8 +642,8 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
             // (a small batch's bands stay in the latency forms)
             const bool small = tab.long_min == 0u && u == kTwinLevels && u < kLatencyLevels &&
                                ((packed.levels >> u) & 1u);
-            if ((small ? launch_latency(c, u, u, 1, all, ka, PHASE_ESCALATED, s, packed)
-                       : launch_unit(c, u, ka, PHASE_ESCALATED, s, packed, units, all)) != LOGAN_OK)
+            if ((small ? launch_latency(c, u, u, all, ka, PHASE_ESCALATED, s, packed)
+                       : launch_unit(c, u, ka, PHASE_ESCALATED, s, packed, all)) != LOGAN_OK)
                 return LOGAN_ECUDA;
             if (!rec(EV_P2E + u, s)) return LOGAN_ECUDA;
             p2_levels |= 1u << u;

@@ -758,6 +758,13 @@ bool packed_level(int level) { return level <= 6; }
 #define LOGAN_PACKED_LATENCY(X) \
     X(0, 1, 32, 2) X(0, 2, 16, 4) X(0, 4, 8, 8) X(1, 1, 32, 4) X(1, 2, 16, 8) X(2, 1, 32, 8)
 
+// Levels 0 and 1, four to a warp, with the general substitution: 64 slots, whose
+// steps cost half as much (3 kbp at +2/-3/-5, X = 20, 1,000 pairs: 0.87 ms with
+// 128 slots, 0.68; lognormal 1.86, 1.41; the 32-bit one-warp form 1.13, 1.55).
+// With +1/-1/-1 unrelated pairs drift to bands of 12 X rows, and moving those to the
+// next window costs more (X = 10: 1.50 ms with 128 slots, 2.02 with 64).
+inline bool half_window(int level, int units, bool unit) { return level <= 1 && units == 4 && !unit; }
+
 // class -> (G, V) of its recording sweep
 #define LOGAN_RECORD_CLASSES(X) X(0, 4, 1) X(1, 8, 1) X(2, 16, 1) X(3, 32, 1) X(4, 32, 2)
 
@@ -825,6 +832,11 @@ cudaError_t launch_packed_level(int level, const KernelArgs& ka, const DiagArgs&
 
 cudaError_t launch_packed_latency(int level, int queue, int units, const KernelArgs& ka,
                                   const DiagArgs& da, int grid, int phase, cudaStream_t s) {
+    if (half_window(level, units, da.unit != 0)) {
+        static_assert(Diag<8, 1, 4>::W == level_window(1) && Diag<8, 1, 4>::W <= mig_rows(0), "window");
+        k_diag16<8, 1, 4, false><<<grid, 128, 0, s>>>(ka, da, level, queue, phase);
+        return cudaGetLastError();
+    }
     switch (latency_form(level, units)) {
 #define CASE(K, U, G, R)                                                                  \
     case 10 * K + U:                                                                      \

@@ -1,0 +1,38 @@
+"""Small batches, whose extensions all take latency forms: on both sides of every
+batch size where the extensions per warp change, at levels 0 to 3, for the
+one-multiply substitution and the general one (whose narrow levels hold half
+the window: bands that outgrow it with and without records).  Results are
+integers: every field equals the oracle's."""
+import numpy as np
+import pytest
+
+from paper_2002_05200_gb300 import logan, synth
+from tests.gpu_common import assert_same, run_gpu, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture()
+def ctx():
+    c = logan.Context(0)
+    yield c
+    c.close()
+
+
+def sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("per_sm", [4, 8, 12, 16, 24])
+@pytest.mark.parametrize("more", [0, 1])
+@pytest.mark.parametrize("scheme", [(1, -1, -1), (2, -3, -5), (2, -2, -2)])
+def test_extensions_per_warp(ctx, scheme, per_sm, more):
+    n = per_sm * sms() // 2 + more
+    b = synth.lognormal_batch(n_pairs=n, median=200, lo=20, hi=700, related_frac=0.8, seed=n, X=50)
+    b.match, b.mismatch, b.gap = scheme
+    b.Xs = np.array([8, 15, 30, 90, 250], np.int32)[np.arange(n) % 5]
+    ref = run_oracle(b)
+    for mig in (64, 0):
+        ctx.set_option(logan.OPT_MIGRATION_MB, mig)
+        assert_same(run_gpu(ctx, b, packed2bit=True), ref, f"{scheme}, {n} pairs, records {mig}")
