@@ -80,6 +80,7 @@ struct logan_ctx {
     // take the latency form; -1 never, -2 automatic
     int64_t long_item = -2;
     uint32_t long_cap = 0xffffffffu;  // and how many of them per level, see ctx_set_long_cap
+    bool paths_follow = false;        // see ctx_set_paths_follow
     // LOGAN_OPT_PACKED16: 1 = run a level in its packed 16-bit form when the
     // call's scoring and X provably fit (see packed16_levels), 0 = never
     int64_t packed16 = 1;
@@ -178,6 +179,8 @@ Layout make_layout(const logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t
 TracebackTiming* logan::ctx_traceback_timing(logan_ctx_t* c) { return &c->tb_timing; }
 
 void logan::ctx_set_matrix_packed(logan_ctx_t* c, uint32_t levels) { c->matrix_packed_last = levels; }
+
+void logan::ctx_set_paths_follow(logan_ctx_t* c, bool on) { c->paths_follow = on; }
 
 void logan::ctx_set_long_cap(logan_ctx_t* c, uint32_t items) { c->long_cap = items; }
 
@@ -369,7 +372,7 @@ AuxSet* aux_for(logan_ctx* c, cudaStream_t s) {
 // class whose start level is at or below it (items only move to wider
 // levels).
 PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int32_t* Xs,
-                           const LevelTable& tab, int64_t force) {
+                           const LevelTable& tab, int64_t force, uint32_t n_items) {
     PackedPlan pk;
     if (!c->packed16) return pk;
     static const int64_t upper[kXClasses] = {15, 35, 75, 150, 300, 700, 2000, int64_t(1) << 29};
@@ -387,6 +390,13 @@ PackedPlan packed16_levels(const logan_ctx* c, Scoring sc, int32_t X, const int3
         }
         if (packed_plan(sc, xmax, &pk.args[l])) pk.levels |= 1u << l;
     }
+    // the few extensions of a tiny batch wait for one step's chain: level 6's block
+    // of four warps has a shorter one than one warp with two virtual lanes, unless
+    // the substitution is one multiply-add (8 pairs of 12 kbp at X = 800, +2/-3/-5
+    // 9.1 and 10.8 ms, 16 pairs 16.0 and 14.4; +1/-1/-1, 8 pairs 11.0 and 7.6)
+    // (what the alignment paths record again runs packed: 1 pair of 12 kbp at X = 800,
+    // +2/-3/-5, with its path 17.5 ms, 23.3 from the block)
+    if (n_items <= 16u && !pk.args[6].unit && !c->paths_follow) pk.levels &= ~(1u << 6);
     // levels 0 and 1 run wider windows packed than in 32 bits: their records
     // need packed readers up to level 2
     if (!((pk.levels >> 2) & 1u)) pk.levels &= ~3u;
@@ -476,7 +486,7 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     tab.long_min = long_item_min(c, 2u * n_pairs);
     const int64_t forced = c->force_level >= 0 ? std::min<int64_t>(c->force_level, maxl) : -1;
     const PackedPlan packed =
-        (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced);
+        (aff || plain) ? PackedPlan{} : packed16_levels(c, sc, X, Xs, tab, forced, n_items);
     // (every item in latency form has the whole GPU, the 32-bit forms do in any case)
     tab.capped = tab.long_min == 0u ? 0u : packed.levels;
     tab.long_cap = std::min(kLongItemsPerSm * uint32_t(c->num_sms), c->long_cap);
@@ -703,7 +713,8 @@ int extend_common(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         uint64_t(uintptr_t(seeds)), uint64_t(uintptr_t(out)), uint64_t(uintptr_t(ws)),
         uint64_t(uintptr_t(stream)), uint64_t(c->force_level), uint64_t(c->max_level),
         uint64_t(c->ring_log2), uint64_t(c->plain_level), uint64_t(c->mig_mb),
-        uint64_t(c->concurrent), uint64_t(c->long_item), uint64_t(c->packed16)};
+        uint64_t(c->concurrent), uint64_t(c->long_item), uint64_t(c->packed16),
+        uint64_t(c->paths_follow)};
     for (const logan_seqs_t* p : {A, B}) {
         key.push_back(uint64_t(uintptr_t(p->bases)));
         key.push_back(uint64_t(uintptr_t(p->offsets)));

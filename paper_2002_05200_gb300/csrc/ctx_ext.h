@@ -31,6 +31,10 @@ void ctx_set_matrix_packed(logan_ctx_t* c, uint32_t levels);
 // knows what else is in flight.
 void ctx_set_long_cap(logan_ctx_t* c, uint32_t items);
 
+// Whether the coming extension's results are swept again for their paths (by
+// the packed recording forms, where a packed level finished them).
+void ctx_set_paths_follow(logan_ctx_t* c, bool on);
+
 // Device views into the workspace of a finished logan_extend_batch call
 // with the same pools and pair count: the 2-bit words of both pools, the
 // split items (two per pair, left first), every item's result (best cell,

@@ -985,9 +985,12 @@ extern "C" int logan_traceback_batch(logan_ctx_t* ctx, const logan_seqs_t* A,
         if (rc == LOGAN_OK && !S.ok) rc = LOGAN_ENOMEM;
         // step 1: the batch pipeline (best cells, cells, packed pools, items)
         clk.mark(TbClock::START, s);
-        if (rc == LOGAN_OK)
+        if (rc == LOGAN_OK) {
+            ctx_set_paths_follow(ctx, true);
             rc = logan_extend_batch(ctx, A, B, seeds, n_pairs, match, mismatch, gap, X,
                                     X_per_pair, ws, ws_bytes, res, stream);
+            ctx_set_paths_follow(ctx, false);
+        }
         clk.mark(TbClock::EXT_END, s);
         if (rc == LOGAN_OK) {
             ExtensionViews v;

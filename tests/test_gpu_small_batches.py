@@ -36,3 +36,15 @@ def test_extensions_per_warp(ctx, scheme, per_sm, more):
     for mig in (64, 0):
         ctx.set_option(logan.OPT_MIGRATION_MB, mig)
         assert_same(run_gpu(ctx, b, packed2bit=True), ref, f"{scheme}, {n} pairs, records {mig}")
+
+
+@pytest.mark.parametrize("n", [1, 8, 9])
+@pytest.mark.parametrize("scheme", [(1, -1, -1), (2, -3, -5)])
+def test_tiny_batches_of_wide_bands(ctx, scheme, n):
+    # level 6 in a block or in one warp, its records to and from the others
+    b = synth.lognormal_batch(n_pairs=n, median=6000, lo=2000, hi=12_000, related_frac=0.5, seed=n, X=50)
+    b.match, b.mismatch, b.gap = scheme
+    for X, level in ((800, -1), (200, 5)):
+        b.X = X
+        ctx.set_option(logan.OPT_FORCE_LEVEL, level)
+        assert_same(run_gpu(ctx, b, packed2bit=True), run_oracle(b), f"{scheme}, {n} pairs, X {X}")
