@@ -6,8 +6,10 @@ integers: every field equals the oracle's."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2002_05200_gb300 import logan, synth
 from tests.gpu_common import assert_same, run_gpu, run_oracle
+from tests.test_gpu_matrix import run_matrix
 
 pytestmark = pytest.mark.gpu
 
@@ -48,3 +50,16 @@ def test_tiny_batches_of_wide_bands(ctx, scheme, n):
         b.X = X
         ctx.set_option(logan.OPT_FORCE_LEVEL, level)
         assert_same(run_gpu(ctx, b, packed2bit=True), run_oracle(b), f"{scheme}, {n} pairs, X {X}")
+
+
+@pytest.mark.parametrize("X,ge", [(219, -1), (220, -1), (439, -2), (440, -2)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_few_proteins_with_wide_bands(ctx, X, ge, more):
+    # the matrix call's windows in 32 bits: few extensions whose bands are wide
+    n = 8 * sms() + more
+    b = synth.protein_pairs(n, lo=20, hi=400, seed=X)
+    b.X = X
+    got = run_matrix(ctx, b, synth.BLOSUM62, -11, ge)
+    few = more == 0 and X >= 220 * -ge
+    assert (ctx.get_option(logan.OPT_MATRIX_PACKED) == 0) == few
+    assert_same(got, oracle.run_batch_matrix(b, synth.BLOSUM62, -11, ge)[0], f"{n} pairs, X {X}")
