@@ -461,10 +461,10 @@ class Context:
         n = ctypes.c_uint64()
         cr = reads.c()
         args = (self._h, ctypes.byref(cr), k, min_freq, max_freq, min_shared)
-        # one call with room for 32 candidates a read (96 MiB at most); only a
-        # read set with more runs a second one at the size that the first
-        # returned
-        cap = max(1024, min(32 * reads.count, 1 << 22))
+        # one call with room for 32 candidates a read (16 in large sets, 1.5 GiB
+        # at most); only a read set with more runs a second one at the size that
+        # the first returned
+        cap = max(1024, min(32 * reads.count, max(1 << 22, 16 * reads.count), 1 << 26))
         while True:
             out = torch.empty((cap, 6), dtype=torch.int32, device=f"cuda:{self.device}")
             _check(lib().logan_overlap_candidates(*args, out.data_ptr(), cap, ctypes.byref(n),
