@@ -50,7 +50,7 @@ METRIC = "X-drop GCUPS (computed cells), batched vs plain launch; serving p50/p9
 PROFILED = {"level": 2, "bytes": 113.513984e6 + 9.392128e6, "items": 48_000,
             "fma_share": 3672597380 / 11914807158,
             "sources": ("xdrop_diag16.cu", "diag16.cuh", "logan_dev.cuh", "internal.h"),
-            "sha1": "7860fcedec66da8efece5639c0ee55a340a6af9d"}
+            "sha1": "540be913943d1953e74f9fc4a1717f55bb934adf"}
 OPS_PER_CELL_AFFINE = 12  # Gotoh per cell: compare, diag add, E: 2 adds + max, F: 2 adds + max, 2 max, X-drop compare, select
 # The scope table's count for the linear recurrence, per cell: substitution
 # select, diag + substitution, max(up, left), + gap and max with the diagonal

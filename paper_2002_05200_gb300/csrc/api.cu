@@ -539,7 +539,6 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
     ka.sc = sc;
     ka.one = 1;
     for (int k = 0; k < 16; ++k) ka.pw[k] = 1u << (31 - 2 * k);
-    for (int k = 0; k < 16; ++k) ka.pw16[k] = 1u << (15 - k);
     for (int l = 0; l < kNumLevels; ++l) {
         ka.next_level[l] = c->next_level[l];
         ka.mig_cap[l] = L.mig_cap[l];

@@ -30,9 +30,6 @@ struct KernelArgs {
     // pw[k] = 2^(31 - 2k): multiplying a 2-bit-per-row flag word by it moves
     // row k's flag to the sign bit (a multiply-add, FMA pipe)
     uint32_t pw[16];
-    // pw16[h] = 2^(15 - h): moves bits h and h + 16 of a row mask to bits 15
-    // and 31 (the halves' top bits) as a multiply-add
-    uint32_t pw16[16];
     // level an item goes to when its band outgrows level k (kNumLevels = ring)
     int8_t next_level[kNumLevels];
     // migration records written by level k (nullptr or cap 0: restart instead)
