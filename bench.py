@@ -47,8 +47,8 @@ METRIC = "X-drop GCUPS (computed cells), batched vs plain launch; serving p50/p9
 #             FMA pipe (IMAD, from sass__inst_executed_per_opcode), the rest
 #             going to the ALU pipe or to pipes that are not near a limit.
 # Reported only while the kernel's sources are the ones captured.
-PROFILED = {"level": 2, "bytes": 113.513984e6 + 9.392128e6, "items": 48_000,
-            "fma_share": 3672597380 / 11914807158,
+PROFILED = {"level": 2, "bytes": 113.391872e6 + 9.102848e6, "items": 48_000,
+            "fma_share": 3674791879 / 11921996529,
             "sources": ("xdrop_diag16.cu", "diag16.cuh", "logan_dev.cuh", "internal.h"),
             "sha1": "540be913943d1953e74f9fc4a1717f55bb934adf"}
 OPS_PER_CELL_AFFINE = 12  # Gotoh per cell: compare, diag add, E: 2 adds + max, F: 2 adds + max, 2 max, X-drop compare, select

@@ -366,7 +366,7 @@ AuxSet* aux_for(logan_ctx* c, cudaStream_t s) {
 }
 
 // Levels that run in their packed 16-bit form in this call: those with a
-// packed kernel whose bounds (xdrop_diag16.cu) hold for the scoring and the
+// packed kernel whose bounds (diag_plan.h) hold for the scoring and the
 // largest X that can reach the level -- the scalar X when there is no
 // per-pair X and no forced start level, else the upper bound of every X
 // class whose start level is at or below it (items only move to wider
@@ -606,8 +606,8 @@ int run_pipeline(logan_ctx* c, const logan_seqs_t* A, const logan_seqs_t* B,
         ++launches;
     } else {
         // phase 1: every queue's binned items; the queues share no entry, so
-        // they run concurrently on their own streams, the latency forms
-        // (long items) first
+        // they run concurrently on their own streams, the latency forms of
+        // levels 0 to 3 (long items) first, level 4's beside its own launch
         AuxSet* ax = c->concurrent ? aux_for(c, s) : nullptr;
         if (ax && cudaEventRecord(ax->fork, s) != cudaSuccess) return LOGAN_ECUDA;
         for (int k = 0; k < kUnits; ++k) {

@@ -185,7 +185,7 @@ __global__ void k_bin_hist(const Item* __restrict__ items, uint32_t n, LevelTabl
 // A few kilobytes between two kernels, so its own latency is its cost: the
 // queues one after the other, 15 block barriers each, took 12.4 us (2.7 now); with
 // warp scans, 16-byte validation loads and no blocks beyond a small batch's
-// items, 1,000 pairs of 1 kbp take 482 us instead of 579, 8 of 2 kbp 350
+// items, 1,000 pairs of 2 kbp take 482 us instead of 579, 8 of them 350
 // instead of 354.
 // one block, a warp per queue: exclusive scan of the bucket counts (longest
 // bucket first, four per lane) -> cursors; queue sizes -> counters (the
