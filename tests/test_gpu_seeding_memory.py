@@ -1,5 +1,5 @@
-"""What overlap_candidates holds on to: the result's own size (at most twice it),
-and a first buffer that does not grow with the read set without end."""
+"""What overlap_candidates holds on to: the result's own size (twice it or 4 MiB
+more at most), and a first buffer that does not grow with the read set without end."""
 import numpy as np
 import pytest
 
@@ -18,12 +18,13 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("n_reads,glen", [(3, 300000), (60, 60000), (120, 3000)])
+@pytest.mark.parametrize("n_reads,glen", [(3, 300000), (120, 3000), (20000, 1000000), (20000, 10000000)])
 def test_result_storage(ctx, n_reads, glen):
     reads = genome_reads(np.random.default_rng(n_reads), n_reads, glen)
     got = ctx.overlap_candidates(device_pool(reads), 15, 2, 8, 1)
     assert got.is_contiguous() and got.shape[1] == 6
-    assert got.untyped_storage().nbytes() <= 2 * ROW * got.shape[0]
+    held, n = got.untyped_storage().nbytes(), got.shape[0]
+    assert held <= max(2 * ROW * n, ROW * n + (4 << 20))
 
 
 def test_first_buffer_of_a_large_read_set(ctx):
