@@ -481,6 +481,9 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     range: 32 * max(D, o + r + 1) + 64 in place
                                     of 32 * D in the second bound;
                                     otherwise, or with 0, the 32-bit form.
+                                    (Level 6 in batches of up to 16 extensions and
+                                    the matrix call with few extensions of wide bands
+                                    may run 32 bits where that is faster.)
                                     Results are identical either way. */
 #define LOGAN_OPT_AFFINE_PACKED 12 /* read-only: bit l set when affine window
                                     level l (64, 128, 256, 512 rows) ran in

@@ -289,9 +289,9 @@ inline int blocks_for_items(const KernelArgs& ka, int units, int most) {
 // Items of a level that take its packed latency form beside the others, at most:
 // two for each of the four warps per SM that the launch below has.  With more the
 // longest stay (whole length buckets) and the rest run several to a warp:
-// 3,000 pairs of 200 kbp, all long, took 266 ms four to an SM and take 62 several to a
-// warp (32-bit latency form with the whole GPU: 194); 1,216 extensions of
-// one length are about even.
+// 3,000 pairs of 200 kbp, all long, X = 50, took 266 ms four to an SM and take 76 with
+// this (32-bit latency form with the whole GPU: 192); 1,216 extensions of one
+// length are about even.
 constexpr uint32_t kLongItemsPerSm = 8;
 
 // The latency form of `level`.  all: it runs every item of the level; else the
