@@ -479,7 +479,8 @@ int logan_extend_batch_noalloc(logan_ctx_t *ctx, const logan_seqs_t *seqsA,
                                     with the gap extension for |gap| and, o =
                                     |gap_open|, r = the substitution scores'
                                     range: 32 * max(D, o + r + 1) + 64 in place
-                                    of 32 * D in the second bound;
+                                    of 32 * D in the second bound, 2*|gap| more
+                                    inside the third's parentheses;
                                     otherwise, or with 0, the 32-bit form.
                                     (Level 6 in batches of up to 16 extensions and
                                     the matrix call with few extensions of wide bands
